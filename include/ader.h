@@ -52,7 +52,10 @@ typedef enum {
 typedef enum { ADER_SCHEME_DG = 0, ADER_SCHEME_WENO_FV = 1 } ader_scheme;
 
 typedef enum {
-  ADER_PREC_FP64 = 0,            /* whole path in FP64 */
+  ADER_PREC_FP64 = 0,            /* FP64 accuracy throughout; the 1D Euler predictor of N >= 1
+                                    runs its sweeps in fixed point with 57 to 61 fraction bits
+                                    below each cell's largest values (cells that do not fit,
+                                    and gamma > 2, in FP64), rounded to FP64 once */
   ADER_PREC_FP32_PREDICTOR = 1,  /* Picard in FP32, then fp64_sweeps FP64 sweeps; rest FP64 */
   ADER_PREC_FF_PREDICTOR = 2,    /* Picard and predictor epilogue in float-float (~48 bits,
                                     FP32 pipes); corrector and CFL in FP64 */
@@ -368,7 +371,8 @@ ader_status ader_get_troubled(ader_ctx* ctx, int32_t* flags_dev, int64_t count);
  * Autotuning of launch shapes (no counterpart in the paper).
  * ------------------------------------------------------------------------- */
 typedef struct {
-  int predict_cells_per_block;  /* predictor tile: 16, 32 or 64 cells x (N+1) threads */
+  int predict_cells_per_block;  /* predictor tile: 16, 32 or 64 cells x (N+1) threads; the FP64
+                                   form's fixed-point kernel: 2, 4 or 8 warps of 32 / (N+1) cells */
   int face_cells_per_block;     /* interface/update tile: 32 or 64 cells per 256 threads */
   int graph_steps;              /* time steps per CUDA-graph replay in ader_solve (even, 2..64) */
   double predict_ms;            /* measured per launch for the chosen shape (autotune only) */

@@ -184,6 +184,8 @@ PredictParams make_predict(const ader_ctx* c, const double* u_nodal, const StepP
   p.sp = sp;
   p.ops = c->basis.d;
   p.opf = c->basis.f;
+  p.opi = c->basis.i;
+  p.fix = set_fx_gamma(p.gamma, &p.opi) ? 1 : 0;
   return p;
 }
 

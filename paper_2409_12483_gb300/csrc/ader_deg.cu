@@ -2,6 +2,7 @@
 // plain launchers.  Compiled once per degree with -DADER_DEG=<0..7>, so the
 // degrees build in parallel and each kernel is fully unrolled for its N.
 #include "ader_kernels.cuh"
+#include "ader_fix.cuh"
 #include "ader_incr.cuh"
 #include "ader_source.cuh"
 #include "ader_limiter.cuh"
@@ -89,6 +90,53 @@ cudaError_t prepare_cpb() {
   }
 }
 
+// The FP64 form runs in fixed point (ader_fix.cuh) from N = 1, except for a given
+// q (from_q: only the epilogue) and an adiabatic index outside its tables; the
+// tuned cells per block choose its warps per block: 2, 4 or 8 for 16, 32 or 64.
+template <int CPB>
+cudaError_t launch_predict_fix(const PredictParams& p, cudaStream_t s) {
+  using C = FixCfg<D, CPB / 8>;
+  const long long blocks = (p.ncells + C::CELLS - 1) / C::CELLS;
+  if (blocks <= 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  // the blocks that fit at once; each takes every grid-th tile
+  const long long resident = 152LL * C::MIN_BLOCKS;
+  const long long grid = blocks < resident ? blocks : resident;
+  predict_fix_kernel<D, C::WPB><<<(unsigned)grid, C::THREADS, C::kSmemBytes, s>>>(p);
+  return cudaGetLastError();
+}
+
+template <int CPB>
+cudaError_t prepare_fix() {
+  using C = FixCfg<D, CPB / 8>;
+  if constexpr (!C::kValid) return cudaSuccess;
+  else
+    return cudaFuncSetAttribute(predict_fix_kernel<D, C::WPB>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes);
+}
+
+
+// the server's batched form
+template <int N>
+cudaError_t launch_fix_multi(const PredictParams& p, const MultiArgs& m, int grid, cudaStream_t s) {
+  using C = FixCfg<N, 4>;
+  if constexpr (!C::kValid) {
+    return cudaErrorInvalidValue;
+  } else {
+    static_assert(C::CELLS == server_fix_cells(N), "the server's tiles");
+    predict_fix_multi_kernel<N, C::WPB><<<(unsigned)grid, C::THREADS, C::kSmemBytes, s>>>(p, m);
+    return cudaGetLastError();
+  }
+}
+
+template <int N>
+cudaError_t prepare_fix_multi() {
+  using C = FixCfg<N, 4>;
+  if constexpr (!C::kValid) return cudaSuccess;
+  else
+    return cudaFuncSetAttribute(predict_fix_multi_kernel<N, C::WPB>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes);
+}
+
 template <int CPB>
 cudaError_t launch_predict_cpb(const PredictParams& p, cudaStream_t s) {
   if constexpr (!PredCfg<D, CPB>::kValid) {
@@ -97,6 +145,9 @@ cudaError_t launch_predict_cpb(const PredictParams& p, cudaStream_t s) {
     using C = PredCfg<D, CPB>;
     const long long blocks = (p.ncells + C::CPB - 1) / C::CPB;
     if (blocks <= 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    if constexpr (D >= 1) {
+      if (p.prec == 0 && !p.from_q && p.fix) return launch_predict_fix<CPB>(p, s);
+    }
     if (p.prec == 1 && !p.from_q)
       predict_kernel<D, 1, CPB><<<(unsigned)blocks, C::THREADS, C::kSmemBytes, s>>>(p);
     else if (p.prec == 2 && !p.from_q && kFFCapped<CPB>)
@@ -214,6 +265,9 @@ cudaError_t launch_face_cf(const FaceParams& p, cudaStream_t s) {
 
 cudaError_t ADER_CAT(prepare_degree_, ADER_DEG)() {
   cudaError_t e;
+  if ((e = prepare_fix<16>()) != cudaSuccess) return e;
+  if ((e = prepare_fix<32>()) != cudaSuccess) return e;
+  if ((e = prepare_fix<64>()) != cudaSuccess) return e;
   if ((e = prepare_cpb<16>()) != cudaSuccess) return e;
   if ((e = prepare_cpb<32>()) != cudaSuccess) return e;
   if ((e = prepare_cpb<64>()) != cudaSuccess) return e;
@@ -249,6 +303,7 @@ cudaError_t ADER_CAT(prepare_degree_, ADER_DEG)() {
                              (int)PredCfg<D, T>::kSmemBytes);
     if (e != cudaSuccess) return e;
   }
+  if ((e = prepare_fix_multi<D>()) != cudaSuccess) return e;
   {
     constexpr int T = server_pred_cells(D);
     e = cudaFuncSetAttribute(predict_incr_multi_kernel<D, T>,
@@ -409,6 +464,7 @@ cudaError_t ADER_CAT(launch_predict_multi_, ADER_DEG)(const PredictParams& p, co
   constexpr int T = server_pred_cells(D);
   using C = PredCfg<D, T>;
   if (grid <= 0) return cudaErrorInvalidValue;
+  if (D >= 1 && p.prec == 0 && p.fix) return launch_fix_multi<D>(p, m, grid, s);
   if (p.prec == 1)
     predict_multi_kernel<D, 1, T><<<(unsigned)grid, C::THREADS, C::kSmemBytes, s>>>(p, m);
   else if (p.prec == 2)

@@ -1,0 +1,177 @@
+// ader_fix.h -- 60-bit fixed-point arithmetic on 32-bit integer multipliers, the
+// number form of the FP64 predictor's inner loop (ader_fix.cuh).
+//
+// GB300 issues 2 FP64 lanes per SM and clock against 64 lanes of 32 x 32 + 64-bit
+// integer multiply-add (mad.wide: 62.7 lanes measured), so a product of two
+// two-limb integers (3 mad.wide) costs a tenth of one DFMA.  Inside one cell the
+// scheme's contractions mix all nodes, so the rounding of a result is set by the
+// largest value of the cell: a common exponent per cell and variable loses
+// nothing against a floating-point significand, and 57 fraction bits below that
+// exponent are more than the 53 of FP64.
+//
+// Numbers: a 64-bit integer X = x 2^f ("frac f"); limbs (h, l) with X = h 2^32 + l
+// and l in [-2^31, 2^31), so that every partial product is a signed 32 x 32 one.
+// A contraction sum_j c_j x_j keeps two 64-bit sums, hh = sum h h and
+// m = sum (h l + l h); the l l terms (below 2^-2 of the last bit kept, of either
+// sign) are left out.  The value of the sum is hh + m 2^-32 in units of 2^64.
+// All functions also compile for the host (the arithmetic is tested there).
+#pragma once
+
+#include <cstdint>
+#include <cstring>
+
+#ifdef __CUDACC__
+#define ADER_HD __host__ __device__ __forceinline__
+#else
+#define ADER_HD inline
+#endif
+
+namespace ader {
+
+typedef long long fxi;
+
+struct Fx2 {
+  int h, l;
+};
+
+// The device forms are PTX: written in C++, (fxi)(int)(x >> 32) becomes an arithmetic
+// 64-bit shift and the product that uses it a 64 x 64-bit one (a flux took 135
+// instructions instead of 75).
+ADER_HD int fx_hi(fxi x) {
+#ifdef __CUDA_ARCH__
+  int h, l;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(l), "=r"(h) : "l"(x));
+  return h;
+#else
+  return (int)(x >> 32);
+#endif
+}
+ADER_HD int fx_lo(fxi x) {
+#ifdef __CUDA_ARCH__
+  int h, l;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(l), "=r"(h) : "l"(x));
+  return l;
+#else
+  return (int)(uint32_t)(uint64_t)x;
+#endif
+}
+ADER_HD fxi fx_join(unsigned h, unsigned l) {
+#ifdef __CUDA_ARCH__
+  fxi x;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(l), "r"(h));
+  return x;
+#else
+  return (fxi)(((uint64_t)h << 32) | l);
+#endif
+}
+
+ADER_HD Fx2 fx_split(fxi x) { return Fx2{fx_hi(x + 0x80000000LL), fx_lo(x)}; }
+
+ADER_HD fxi fx_madw(int a, int b, fxi c) { return (fxi)a * (fxi)b + c; }
+// (x << k) and (x >> k) of the 96-bit number x:lo, the words that stay
+ADER_HD unsigned fx_funnel_l(unsigned lo, unsigned hi, int k) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_l(lo, hi, k);
+#else
+  return (k & 31) ? (hi << (k & 31)) | (lo >> (32 - (k & 31))) : hi;
+#endif
+}
+
+// Sums of a contraction; SH: the left shift of its fold (rounds to nearest).  m is kept
+// in two parts, so that no chain of multiply-adds is longer than the sum.
+struct FxAcc {
+  fxi hh, m, m2;
+};
+template <int SH>
+ADER_HD FxAcc fx_zero() {
+  return FxAcc{0, (fxi)1 << (31 - SH), 0};
+}
+ADER_HD void fx_mac(FxAcc& s, int ch, int cl, const Fx2& x) {
+  s.hh = fx_madw(ch, x.h, s.hh);
+  s.m = fx_madw(ch, x.l, s.m);
+  s.m2 = fx_madw(cl, x.h, s.m2);
+}
+// (hh + m 2^-32) 2^SH
+template <int SH>
+ADER_HD fxi fx_fold(const FxAcc& s) {
+  const fxi m = s.m + s.m2;
+  const fxi t = s.hh + (fxi)fx_hi(m);
+  if constexpr (SH == 0) {
+    return t;
+  } else {
+    const unsigned w = (unsigned)fx_lo(t);
+    return fx_join(fx_funnel_l(w, (unsigned)fx_hi(t), SH),
+                   fx_funnel_l((unsigned)fx_lo(m), w, SH));
+  }
+}
+// the same with a run-time shift in [0, 31]; the rounding (1 << 31 - sh) is the
+// caller's initial m
+ADER_HD fxi fx_fold_var(const FxAcc& s, int sh) {
+  const fxi m = s.m + s.m2;
+  const fxi t = s.hh + (fxi)fx_hi(m);
+  const unsigned w = (unsigned)fx_lo(t);
+  return fx_join(fx_funnel_l(w, (unsigned)fx_hi(t), sh),
+                 fx_funnel_l((unsigned)fx_lo(m), w, sh));
+}
+
+// Formats of the predictor, in the cell's units (|q| < 2): rho and m at frac 61, E
+// at frac 57; fluxes and everything that enters a contraction below 2^60 (frac 57).
+constexpr int kFxF = 57;
+constexpr int kFxM = 61;
+// log2 bounds of the row sums of |k~|, |psi| (both ends) and |D~ / w|, by degree:
+// a table entry is stored at frac 62 - bound, so the high limbs of a row sum to
+// less than 2^30 and no 64-bit sum can overflow.
+constexpr int kFxSK[8] = {0, 2, 4, 5, 6, 6, 7, 8};
+constexpr int kFxSP[8] = {1, 1, 2, 2, 2, 2, 3, 3};
+constexpr int kFxSV[8] = {0, 2, 3, 4, 5, 5, 5, 6};
+
+// One 1D Euler flux in fixed point: rho, m (frac 61), E (frac 57), all below 2 in
+// magnitude, to F0 = m, F1 = m u + p and F2 = (E + p) u at frac 57.  g2h, g2l:
+// (gamma - 1) / 2 <= 1/2 at frac 62.  `bad` collects nonzero bits when rho is not
+// above 1/8 or |u| or |F2| leaves 2 or 8 (then |m u| < 4, |p| < 4, |E + p| < 6).
+//   r   = 1 / rho to 2^-28: float reciprocal of the high limb, one Newton step;
+//   u   = u0 + (m - rho u0) r, u0 = m r at frac 28: the remainder is below 2^-26 and
+//         exact to 2^-57, so 32-bit arithmetic modulo 2^32 gives it at frac 57;
+//   the products' l l terms, left out, stay below 2^-56 (rms 2^-57).
+ADER_HD void fx_flux(fxi rho, fxi m, fxi E, int g2h, int g2l, fxi& F0, fxi& F1, fxi& F2,
+                     unsigned& bad) {
+  const Fx2 R = fx_split(rho), M = fx_split(m);
+  bad |= (unsigned)(R.h - 0x4100000) & 0x80000000u;
+#ifdef __CUDA_ARCH__
+  float rf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"((float)R.h));
+  const int r0 = __float2int_rn(rf * 0x1p57f);  // frac 28
+#else
+  const int r0 = R.h < 0x4100000 ? 0 : (int)(0x1p57f * (1.0f / (float)R.h));
+#endif
+  const int nh = (int)(0u - (unsigned)R.h);
+  const fxi e = fx_madw(nh, r0, (fxi)1 << 57);
+  const int es = (int)fx_funnel_l((unsigned)fx_lo(e), (unsigned)fx_hi(e), 24);  // e >> 8
+  const int r1 = r0 + (fx_hi(fx_madw(r0, es, (fxi)1 << 48)) >> 17);
+  const fxi pu = fx_madw(M.h, r1, (fxi)1 << 28);  // frac 57
+  bad |= ((unsigned)fx_hi(pu) + (1u << 26)) & 0xf8000000u;
+  const int u0 = (int)fx_funnel_l((unsigned)fx_lo(pu), (unsigned)fx_hi(pu), 3);  // pu >> 29
+  const unsigned m4 = fx_funnel_l((unsigned)fx_lo(m), (unsigned)fx_hi(m), 28);   // m >> 4
+  const int d = (int)(m4 + (unsigned)nh * (unsigned)u0 -
+                      (unsigned)fx_hi(fx_madw(R.l, u0, (fxi)1 << 31)));
+  const fxi us = fx_madw(d, r1, (fxi)1 << 24);
+  Fx2 U = fx_split(fx_join((unsigned)(fx_hi(us) >> 25),
+                           fx_funnel_l((unsigned)fx_lo(us), (unsigned)fx_hi(us), 7)));
+  U.h = (int)((unsigned)U.h + (unsigned)u0);  // u = u0 + (us >> 25) at frac 60
+  FxAcc a = fx_zero<0>();
+  fx_mac(a, M.h, M.l, U);
+  const fxi mu = fx_fold<0>(a);
+  const Fx2 W = fx_split(E + E - mu);
+  a = fx_zero<2>();
+  fx_mac(a, g2h, g2l, W);
+  const fxi p = fx_fold<2>(a);
+  const Fx2 H = fx_split(E + p);
+  a = fx_zero<4>();
+  fx_mac(a, H.h, H.l, U);
+  F0 = fx_join((unsigned)(fx_hi(m) >> 4), m4);
+  F1 = mu + p;
+  F2 = fx_fold<4>(a);
+  bad |= ((unsigned)fx_hi(F2) + (1u << 28)) & 0xe0000000u;
+}
+
+}  // namespace ader

@@ -601,11 +601,13 @@ __device__ __forceinline__ void epilogue_ff(const PredictParams& P, const ff (&q
 //   2: Picard in float-float (FP64-accurate, FP32 pipes);
 //   3: Picard in FP32 followed by P.sweeps float-float sweeps.
 // The epilogue (traces, volume term) is float-float in forms 2 and 3, FP64 otherwise.
-template <int N, int PREC, int CPB = 32>
+// The fixed-point form (ader_fix.cuh) calls it with blocks of THREADS threads and
+// tiles of CELLS cells that CPB n does not match, for the cells marked in `only`.
+template <int N, int PREC, int CPB = 32, int CELLS = CPB, int THREADS = PredCfg<N, CPB>::THREADS>
 __device__ __forceinline__ void predict_tile(const PredictParams& P, const TileIO& io,
                                              long long tile, double lam, double* smem,
-                                             PredShared<N>& sh) {
-  constexpr int n = N + 1, THREADS = PredCfg<N, CPB>::THREADS;
+                                             PredShared<N>& sh, const int* only = nullptr) {
+  constexpr int n = N + 1;
   double* sg = smem;                        // [CPB][n][n][3]
   double* sfb = smem + CPB * n * n * kM;    // [CPB][n][3]
   double* su = sfb + CPB * n * kM;          // [CPB][n][3] initial data of the tile's cells
@@ -613,8 +615,8 @@ __device__ __forceinline__ void predict_tile(const PredictParams& P, const TileI
 
   const int tid = threadIdx.x;
   const int lc = tid / n, p0 = tid - lc * n;
-  const long long cell = tile * CPB + lc;
-  const bool valid = cell < io.ncells;
+  const long long cell = tile * CELLS + lc;
+  const bool valid = (CELLS == CPB || lc < CELLS) && cell < io.ncells && (!only || only[lc]);
   for (int i = tid; i < 2 * kMaxCpb * 2; i += THREADS) (&s_red[0][0][0])[i] = 0ull;
   if constexpr (PREC != 2) {  // (dt/dx) kappa~ once per block (made visible by the barrier below)
     if (tid < n * n) sh.kr[tid / n][tid % n] = lam * P.ops.kap[tid / n][tid % n];

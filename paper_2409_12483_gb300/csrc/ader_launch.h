@@ -39,6 +39,8 @@ struct PredictParams {
   StepParams sp;
   OpsD ops;
   OpsF opf;
+  OpsI opi;
+  int fix;               // FP64 form: the fixed-point kernel may run (0 < gamma - 1 <= 1)
 };
 
 // Interface flux (Rusanov at every tau node, GL-weighted in time) fused with the
@@ -96,6 +98,9 @@ struct TileItem {
 // kernels' default tiles.
 constexpr int server_pred_cells(int N) { return N == 0 ? 32 : 16; }
 constexpr int kServerFaceCells = 32;
+// the FP64 form's fixed-point kernel (N >= 1, PredictParams::fix): four warps of
+// 32 / (N + 1) cells
+constexpr int server_fix_cells(int N) { return 4 * (32 / (N + 1)); }
 
 struct MultiArgs {
   const SlotDesc* slots;

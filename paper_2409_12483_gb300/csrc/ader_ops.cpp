@@ -1,6 +1,8 @@
 // ader_ops.cpp -- host construction of the operator tables (see ader_ops.h).
 #include "ader_ops.h"
 
+#include "ader_fix.h"
+
 #include <cmath>
 #include <cstring>
 
@@ -154,6 +156,20 @@ ld factorial_ratio(int j, int a) {  // j! / (j-a)!
 
 }  // namespace
 
+void split_fx(long double x, int frac, int out[2]) {
+  const Fx2 v = fx_split((fxi)llroundl(ldexpl(x, frac)));
+  out[0] = v.h;
+  out[1] = v.l;
+}
+
+bool set_fx_gamma(double gamma, OpsI* o) {
+  // the same difference the FP64 kernels use
+  const double gm1 = gamma - 1.0;
+  if (!(gm1 > 0.0) || !(gm1 <= 1.0)) return false;
+  split_fx(0.5L * (ld)gm1, 62, o->g2);
+  return true;
+}
+
 int build_basis(int N, bool weno, Basis* out) {
   if (!out || N < 0 || N > kMaxDeg) return -1;
   std::memset(out, 0, sizeof(*out));
@@ -211,7 +227,28 @@ int build_basis(int N, bool weno, Basis* out) {
       split_ff(D[l][k], &f.kt[k][l], &f.ktlo[k][l]);
       split_ff(kap[k][l], &f.kap[k][l], &f.kaplo[k][l]);
       split_ff(vt, &f.vt[k][l], &f.vtlo[k][l]);
+      split_fx(D[l][k], 62 - kFxSK[N], out->i.kt[k][l]);
+      split_fx(vt, 62 - kFxSV[N], out->i.vt[k][l]);
     }
+    split_fx(w[k], 62, out->i.w[k]);
+  }
+  for (int k = 0; k < (n + 1) / 2; ++k) {
+    const bool mid = 2 * k + 1 == n;
+    split_fx(mid ? ph1[k] : (ph1[k] + ph0[k]) / 2, 63 - kFxSP[N], out->i.pa[k]);
+    split_fx(mid ? 0 : (ph1[k] - ph0[k]) / 2, 63 - kFxSP[N], out->i.pb[k]);
+  }
+  // the row sums stay inside the bounds the fixed-point sums rely on
+  for (int k = 0; k < n; ++k) {
+    ld sk = 0, sv = 0, s0 = 0, s1 = 0;
+    for (int l = 0; l < n; ++l) {
+      sk += fabsl(D[l][k]);
+      sv += fabsl(w[l] * D[k][l] / w[k]);
+      s0 += fabsl(ph0[l]);
+      s1 += fabsl(ph1[l]);
+    }
+    if (sk > ldexpl(1, kFxSK[N]) || sv > ldexpl(1, kFxSV[N]) || s0 > ldexpl(1, kFxSP[N]) ||
+        s1 > ldexpl(1, kFxSP[N]))
+      return -7;
   }
   // k~ (= Dphi^T) in even/odd form
   {
@@ -226,6 +263,8 @@ int build_basis(int N, bool weno, Basis* out) {
         d.ksb[p][q] = (double)b;
         out->f.ksa[p][q] = (float)a;
         out->f.ksb[p][q] = (float)b;
+        split_fx(a, 63 - kFxSK[N], out->i.ka[p][q]);
+        split_fx(b, 63 - kFxSK[N], out->i.kb[p][q]);
       }
   }
   // subcell projection (Sec. 1.4): P_jk = Ns int_{j/Ns}^{(j+1)/Ns} phi_k = sum_q w_q phi_k((j+xi_q)/Ns)

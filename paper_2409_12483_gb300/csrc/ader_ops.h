@@ -57,6 +57,19 @@ struct OpsF {
   float ksa[kMaxH][kMaxH], ksb[kMaxH][kMaxH];
 };
 
+// Fixed-point tables (ader_fix.h): entries as two-limb integers (h, l) at frac
+// 62 - kFxSK / kFxSV[N] (k~, D~ / w), 62 (w, (gamma - 1) / 2); the even/odd forms
+// (half the row sums) at frac 63 - kFxSK / kFxSP[N]: ka, kb as ksa, ksb of OpsD, and
+// pa[k] = (phi_k(1) + phi_k(0)) / 2, pb[k] = (phi_k(1) - phi_k(0)) / 2 for k < n / 2,
+// pa of the middle node of odd n phi_k(1).
+struct OpsI {
+  int kt[kMaxN][kMaxN][2];
+  int ka[kMaxH][kMaxH][2], kb[kMaxH][kMaxH][2];
+  int pa[kMaxH][2], pb[kMaxH][2], w[kMaxN][2];
+  int vt[kMaxN][kMaxN][2];
+  int g2[2];  // (gamma - 1) / 2, set with the options
+};
+
 // WENO tables for even N (order N+1), three stencils of N+1 cells.
 struct WenoOps {
   int shift[3];                   // first cell of each stencil relative to i
@@ -75,12 +88,19 @@ struct Basis {
   int N = 0, n = 1, Ns = 1;
   OpsD d{};
   OpsF f{};
+  OpsI i{};
   WenoOps weno{};
   // extra host-only tables for inspection
   double dphi[kMaxN][kMaxN]{};    // dphi[k][l] = phi_k'(xi_l)
   double dtil[kMaxN][kMaxN]{};    // D~[k][l]
   double R[kMaxN][kMaxNs]{};      // (P^T P)^-1 P^T: DG coefficients from subcell averages (eq. r_operator)
 };
+
+// x as limbs at the given frac (round to nearest); |x| 2^frac < 2^62.
+void split_fx(long double x, int frac, int out[2]);
+
+// (gamma - 1) / 2 at frac 62; false when the fixed-point form cannot hold it.
+bool set_fx_gamma(double gamma, OpsI* o);
 
 // Returns 0 on success.  weno != 0 also builds the WENO tables (N even, 2 <= N).
 int build_basis(int N, bool weno, Basis* out);

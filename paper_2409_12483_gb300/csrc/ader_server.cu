@@ -178,6 +178,8 @@ PredictParams server_predict_params(const ader_server* srv, int N) {
   p.tolf = (float)p.tol;
   p.ops = srv->basis[N].d;
   p.opf = srv->basis[N].f;
+  p.opi = srv->basis[N].i;
+  p.fix = set_fx_gamma(p.gamma, &p.opi) ? 1 : 0;
   return p;
 }
 
@@ -246,13 +248,15 @@ ader_status admit(ader_server* srv, Req* r, int slot_id, double now) {
 
 ader_status rebuild(ader_server* srv) {
   std::vector<TileItem> items;
+  OpsI oi;
+  const bool fix = srv->opt.precision == ADER_PREC_FP64 && set_fx_gamma(srv->opt.gamma, &oi);
   for (int N = 0; N <= kMaxDeg; ++N) {
     auto& L = srv->lists[N];
     L.pred_off = (long long)items.size();
     for (size_t s = 0; s < srv->slots.size(); ++s) {
       const Req* r = srv->slots[s].req;
       if (!r || r->degree != N) continue;
-      const long long T = server_pred_cells(N);
+      const long long T = fix && N >= 1 ? server_fix_cells(N) : server_pred_cells(N);
       for (long long t = 0; t < (r->ncells + T - 1) / T; ++t) items.push_back({(int)s, (int)t});
     }
     L.pred_n = (long long)items.size() - L.pred_off;
