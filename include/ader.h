@@ -52,8 +52,8 @@ typedef enum {
 typedef enum { ADER_SCHEME_DG = 0, ADER_SCHEME_WENO_FV = 1 } ader_scheme;
 
 typedef enum {
-  ADER_PREC_FP64 = 0,            /* FP64 accuracy throughout; the 1D Euler predictor of N >= 1
-                                    runs its sweeps in fixed point with 57 to 61 fraction bits
+  ADER_PREC_FP64 = 0,            /* FP64 accuracy throughout; the Euler predictors of N >= 1 (3D:
+                                    N <= 4) run their sweeps in fixed point with 57 to 61 fraction bits
                                     below each cell's largest values (cells that do not fit,
                                     and gamma > 2, in FP64), rounded to FP64 once */
   ADER_PREC_FP32_PREDICTOR = 1,  /* Picard in FP32, then fp64_sweeps FP64 sweeps; rest FP64 */

@@ -351,6 +351,9 @@ ader_status enqueue_step2d(ader_ctx* ctx, const double* src, double* dst, const 
   p.inv_dy = 1.0 / ctx->dy;
   p.sp = sp;
   p.ops = ctx->basis.d;
+  p.opi = ctx->basis.i;
+  p.fix = set_fx_gamma(p.gamma, &p.opi) ? 1 : 0;
+  p.tolf = (float)p.tol;
   CK(do_predict2d(ctx->N, p, ctx->stream));
   if (ev) CK(cudaEventRecordWithFlags(ev[2], ctx->stream, cudaEventRecordExternal));
   Face2DParams f{};
@@ -392,6 +395,9 @@ ader_status enqueue_step3d(ader_ctx* ctx, const double* src, double* dst, const 
   p.inv_dz = 1.0 / ctx->dz;
   p.sp = sp;
   p.ops = ctx->basis.d;
+  p.opi = ctx->basis.i;
+  p.fix = set_fx_gamma(p.gamma, &p.opi) ? 1 : 0;
+  p.tolf = (float)p.tol;
   CK(do_predict3d(ctx->N, p, ctx->stream));
   if (ev) CK(cudaEventRecordWithFlags(ev[2], ctx->stream, cudaEventRecordExternal));
   Face3DParams f{};

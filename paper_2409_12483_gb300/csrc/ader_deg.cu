@@ -8,6 +8,7 @@
 #include "ader_limiter.cuh"
 #include "ader_kernels2d.cuh"
 #include "ader_kernels3d.cuh"
+#include "ader_fixd.cuh"
 #include "ader_tracer.cuh"
 
 #ifndef ADER_DEG
@@ -38,9 +39,33 @@ int flat_threads(long long items) { return items >= 152LL * 4 * 256 ? 256 : 64; 
 // two blocks per SM, else the small one (the same shape when they coincide).
 bool use_big_blocks(long long ncells, int big_cpb) { return ncells >= 152LL * 2 * big_cpb; }
 
+// The fixed-point predictors (ader_fixd.cuh), from N = 1 where one thread per
+// space-time node fits a block.
+template <int DIM, int T, typename Params>
+cudaError_t launch_fixd(const Params& p, cudaStream_t s) {
+  using C = FixDCfg<DIM, D, T>;
+  if constexpr (!C::kValid) {
+    return cudaErrorInvalidConfiguration;
+  } else {
+    predict_fixd_kernel<DIM, D, T><<<grid_for(p.ncells, C::CPB, 0x7fffffffLL), C::THREADS,
+                                     fixd_smem_bytes<DIM, D, T>(), s>>>(p);
+    return cudaGetLastError();
+  }
+}
+
+template <int DIM, int T>
+cudaError_t prepare_fixd() {
+  if constexpr (!FixDCfg<DIM, D, T>::kValid) return cudaSuccess;
+  else
+    return cudaFuncSetAttribute(predict_fixd_kernel<DIM, D, T>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)fixd_smem_bytes<DIM, D, T>());
+}
+
 template <int T>
 cudaError_t launch_predict2d_shape(const Predict2DParams& p, cudaStream_t s) {
   using C = Pred2Cfg<D, T>;
+  if (FixDCfg<2, D, T>::kValid && p.fix) return launch_fixd<2, T>(p, s);
   predict2d_kernel<D, T><<<grid_for(p.ncells, C::CPB, 0x7fffffffLL), C::THREADS, 0, s>>>(p);
   return cudaGetLastError();
 }
@@ -271,6 +296,12 @@ cudaError_t ADER_CAT(prepare_degree_, ADER_DEG)() {
   if ((e = prepare_cpb<16>()) != cudaSuccess) return e;
   if ((e = prepare_cpb<32>()) != cudaSuccess) return e;
   if ((e = prepare_cpb<64>()) != cudaSuccess) return e;
+  if ((e = prepare_fixd<2, 256>()) != cudaSuccess) return e;
+  if ((e = prepare_fixd<2, 64>()) != cudaSuccess) return e;
+  if constexpr (D <= kMax3DLowDeg) {
+    if ((e = prepare_fixd<3, 256>()) != cudaSuccess) return e;
+    if ((e = prepare_fixd<3, 64>()) != cudaSuccess) return e;
+  }
   if ((e = prepare_src_cpb<16>()) != cudaSuccess) return e;
   if ((e = prepare_src_cpb<32>()) != cudaSuccess) return e;
   if constexpr (D <= kMax3DDeg) {  // 3D kernels with more than 48 KB of shared memory
@@ -373,6 +404,9 @@ cudaError_t ADER_CAT(launch_predict3d_, ADER_DEG)(const Predict3DParams& p, cuda
   if constexpr (D <= kMax3DLowDeg) {
     using B = Pred3Cfg<D, 256>;
     using S = Pred3Cfg<D, 64>;
+    if (FixDCfg<3, D, 256>::kValid && p.fix)
+      return B::CPB != S::CPB && !use_big_blocks(p.ncells, B::CPB) ? launch_fixd<3, 64>(p, s)
+                                                                   : launch_fixd<3, 256>(p, s);
     if (B::CPB != S::CPB && !use_big_blocks(p.ncells, B::CPB))
       predict3d_kernel<D, 64><<<grid_for(p.ncells, S::CPB, 0x7fffffffLL), S::THREADS, 0, s>>>(p);
     else

@@ -105,11 +105,12 @@ ADER_HD fxi fx_fold(const FxAcc& s) {
   }
 }
 // the same with a run-time shift in [0, 31]; the rounding (1 << 31 - sh) is the
-// caller's initial m
-ADER_HD fxi fx_fold_var(const FxAcc& s, int sh) {
+// caller's initial m; top: the high word before the shift
+ADER_HD fxi fx_fold_var(const FxAcc& s, int sh, int* top = nullptr) {
   const fxi m = s.m + s.m2;
   const fxi t = s.hh + (fxi)fx_hi(m);
   const unsigned w = (unsigned)fx_lo(t);
+  if (top) *top = fx_hi(t);
   return fx_join(fx_funnel_l(w, (unsigned)fx_hi(t), sh),
                  fx_funnel_l((unsigned)fx_lo(m), w, sh));
 }
@@ -125,17 +126,18 @@ constexpr int kFxSK[8] = {0, 2, 4, 5, 6, 6, 7, 8};
 constexpr int kFxSP[8] = {1, 1, 2, 2, 2, 2, 3, 3};
 constexpr int kFxSV[8] = {0, 2, 3, 4, 5, 5, 5, 6};
 
-// One 1D Euler flux in fixed point: rho, m (frac 61), E (frac 57), all below 2 in
-// magnitude, to F0 = m, F1 = m u + p and F2 = (E + p) u at frac 57.  g2h, g2l:
-// (gamma - 1) / 2 <= 1/2 at frac 62.  `bad` collects nonzero bits when rho is not
-// above 1/8 or |u| or |F2| leaves 2 or 8 (then |m u| < 4, |p| < 4, |E + p| < 6).
+// The Euler fluxes of D directions in fixed point: q = (rho, m_1 .. m_D, E), rho and m
+// at frac 61, E at frac 57, all below 2 in magnitude, to F[d] = (m_d, m_j u_d + p
+// (j = d), (E + p) u_d) at frac 57.  g2h, g2l: (gamma - 1) / 2 <= 1/2 at frac 62.  `bad`
+// collects nonzero bits when rho is not above 1/8, a |u_d| leaves 2 or a flux leaves 8.
 //   r   = 1 / rho to 2^-28: float reciprocal of the high limb, one Newton step;
 //   u   = u0 + (m - rho u0) r, u0 = m r at frac 28: the remainder is below 2^-26 and
 //         exact to 2^-57, so 32-bit arithmetic modulo 2^32 gives it at frac 57;
 //   the products' l l terms, left out, stay below 2^-56 (rms 2^-57).
-ADER_HD void fx_flux(fxi rho, fxi m, fxi E, int g2h, int g2l, fxi& F0, fxi& F1, fxi& F2,
-                     unsigned& bad) {
-  const Fx2 R = fx_split(rho), M = fx_split(m);
+template <int D>
+ADER_HD void fx_fluxes(const fxi (&q)[D + 2], int g2h, int g2l, fxi (&F)[D][D + 2],
+                       unsigned& bad) {
+  const Fx2 R = fx_split(q[0]);
   bad |= (unsigned)(R.h - 0x4100000) & 0x80000000u;
 #ifdef __CUDA_ARCH__
   float rf;
@@ -148,30 +150,66 @@ ADER_HD void fx_flux(fxi rho, fxi m, fxi E, int g2h, int g2l, fxi& F0, fxi& F1, 
   const fxi e = fx_madw(nh, r0, (fxi)1 << 57);
   const int es = (int)fx_funnel_l((unsigned)fx_lo(e), (unsigned)fx_hi(e), 24);  // e >> 8
   const int r1 = r0 + (fx_hi(fx_madw(r0, es, (fxi)1 << 48)) >> 17);
-  const fxi pu = fx_madw(M.h, r1, (fxi)1 << 28);  // frac 57
-  bad |= ((unsigned)fx_hi(pu) + (1u << 26)) & 0xf8000000u;
-  const int u0 = (int)fx_funnel_l((unsigned)fx_lo(pu), (unsigned)fx_hi(pu), 3);  // pu >> 29
-  const unsigned m4 = fx_funnel_l((unsigned)fx_lo(m), (unsigned)fx_hi(m), 28);   // m >> 4
-  const int d = (int)(m4 + (unsigned)nh * (unsigned)u0 -
-                      (unsigned)fx_hi(fx_madw(R.l, u0, (fxi)1 << 31)));
-  const fxi us = fx_madw(d, r1, (fxi)1 << 24);
-  Fx2 U = fx_split(fx_join((unsigned)(fx_hi(us) >> 25),
-                           fx_funnel_l((unsigned)fx_lo(us), (unsigned)fx_hi(us), 7)));
-  U.h = (int)((unsigned)U.h + (unsigned)u0);  // u = u0 + (us >> 25) at frac 60
-  FxAcc a = fx_zero<0>();
-  fx_mac(a, M.h, M.l, U);
-  const fxi mu = fx_fold<0>(a);
-  const Fx2 W = fx_split(E + E - mu);
-  a = fx_zero<2>();
-  fx_mac(a, g2h, g2l, W);
+  Fx2 M[D], U[D];
+  unsigned m4[D];
+  fxi W = q[D + 1] + q[D + 1], P[D][D];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+  for (int d = 0; d < D; ++d) {
+    const fxi m = q[1 + d];
+    M[d] = fx_split(m);
+    const fxi pu = fx_madw(M[d].h, r1, (fxi)1 << 28);  // frac 57
+    bad |= ((unsigned)fx_hi(pu) + (1u << 26)) & 0xf8000000u;
+    const int u0 = (int)fx_funnel_l((unsigned)fx_lo(pu), (unsigned)fx_hi(pu), 3);  // pu >> 29
+    m4[d] = fx_funnel_l((unsigned)fx_lo(m), (unsigned)fx_hi(m), 28);               // m >> 4
+    const int rem = (int)(m4[d] + (unsigned)nh * (unsigned)u0 -
+                          (unsigned)fx_hi(fx_madw(R.l, u0, (fxi)1 << 31)));
+    const fxi us = fx_madw(rem, r1, (fxi)1 << 24);
+    U[d] = fx_split(fx_join((unsigned)(fx_hi(us) >> 25),
+                            fx_funnel_l((unsigned)fx_lo(us), (unsigned)fx_hi(us), 7)));
+    U[d].h = (int)((unsigned)U[d].h + (unsigned)u0);  // u0 + (us >> 25) at frac 60
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int i = 0; i <= d; ++i) {
+      FxAcc a = fx_zero<0>();
+      fx_mac(a, M[d].h, M[d].l, U[i]);
+      P[d][i] = fx_fold<0>(a);
+    }
+    W -= P[d][d];
+  }
+  const Fx2 Ws = fx_split(W);
+  FxAcc a = fx_zero<2>();
+  fx_mac(a, g2h, g2l, Ws);
   const fxi p = fx_fold<2>(a);
-  const Fx2 H = fx_split(E + p);
-  a = fx_zero<4>();
-  fx_mac(a, H.h, H.l, U);
-  F0 = fx_join((unsigned)(fx_hi(m) >> 4), m4);
-  F1 = mu + p;
-  F2 = fx_fold<4>(a);
-  bad |= ((unsigned)fx_hi(F2) + (1u << 28)) & 0xe0000000u;
+  const Fx2 H = fx_split(q[D + 1] + p);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+  for (int d = 0; d < D; ++d) {
+    F[d][0] = fx_join((unsigned)(fx_hi(q[1 + d]) >> 4), m4[d]);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int j = 0; j < D; ++j) F[d][1 + j] = j == d ? P[d][d] + p : j < d ? P[d][j] : P[j][d];
+    a = fx_zero<4>();
+    fx_mac(a, H.h, H.l, U[d]);
+    F[d][D + 1] = fx_fold<4>(a);
+    // 1D: |m u| < 4 and |p| < 4 already
+    if (D > 1) bad |= ((unsigned)fx_hi(F[d][1 + d]) + (1u << 28)) & 0xe0000000u;
+    bad |= ((unsigned)fx_hi(F[d][D + 1]) + (1u << 28)) & 0xe0000000u;
+  }
+}
+
+ADER_HD void fx_flux(fxi rho, fxi m, fxi E, int g2h, int g2l, fxi& F0, fxi& F1, fxi& F2,
+                     unsigned& bad) {
+  const fxi q[3] = {rho, m, E};
+  fxi F[1][3];
+  fx_fluxes<1>(q, g2h, g2l, F, bad);
+  F0 = F[0][0];
+  F1 = F[0][1];
+  F2 = F[0][2];
 }
 
 }  // namespace ader

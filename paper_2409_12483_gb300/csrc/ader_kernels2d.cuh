@@ -125,26 +125,19 @@ struct Pred2Shared {
   int go;
 };
 
-template <int N, int T = 256>
-__global__ void __launch_bounds__(Pred2Cfg<N, T>::THREADS, Pred2Cfg<N, T>::MIN_BLOCKS)
-    predict2d_kernel(const __grid_constant__ Predict2DParams P) {
+// One block of cells in FP64; only: the cells to do (null: all), for the cells that
+// the fixed-point form (ader_fixd.cuh) hands over.
+template <int N, int T>
+__device__ __forceinline__ void predict2d_block(const Predict2DParams& P, Pred2Shared<N, T>& sh,
+                                                double dt, const int* only) {
   using C = Pred2Cfg<N, T>;
   constexpr int n = N + 1, NN = C::NN, NST = C::NST, CPB = C::CPB;
-  __shared__ Pred2Shared<N, T> sh;
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    double d = 0.0;
-    sh.go = predictor_step_dt(P.sp, &d, blockIdx.x == 0) ? 1 : 0;
-    sh.dt = d;
-  }
-  __syncthreads();
-  if (!sh.go) return;  // uniform
-  const double dt = sh.dt;
   const double lx = dt * P.sp.inv_dx, ly = dt * P.inv_dy;
   const int lc = tid / NST, node = tid - lc * NST;
   const int p0 = node / NN, p1 = (node / n) % n, p2 = node % n;
   const long long cell = (long long)blockIdx.x * CPB + lc;
-  const bool valid = cell < P.ncells;
+  const bool valid = cell < P.ncells && (!only || only[lc]);
   const OpsD& o = P.ops;
   double uo[kM2], q[kM2];
 #pragma unroll
@@ -180,7 +173,7 @@ __global__ void __launch_bounds__(Pred2Cfg<N, T>::THREADS, Pred2Cfg<N, T>::MIN_B
   const int sk = kPack ? tid - sc * NN : node;
   const int sk1 = kPack ? sk / n : p1, sk2 = kPack ? sk - (sk / n) * n : p2;
   const long long scell = kPack ? (long long)blockIdx.x * CPB + sc : cell;
-  const bool sitem = tid < CPB * NN && scell < P.ncells;
+  const bool sitem = tid < CPB * NN && scell < P.ncells && (!only || only[sc]);
   const int cap = P.fixed_iter > 0 ? P.fixed_iter : P.max_iter;
   for (int it = 0; it < cap; ++it) {
     const bool active = !sh.done[lc];
@@ -350,6 +343,20 @@ __global__ void __launch_bounds__(Pred2Cfg<N, T>::THREADS, Pred2Cfg<N, T>::MIN_B
       rec[4 * NN * kM2 + sk * kM2 + r] = acc;
     }
   }
+}
+
+template <int N, int T = 256>
+__global__ void __launch_bounds__(Pred2Cfg<N, T>::THREADS, Pred2Cfg<N, T>::MIN_BLOCKS)
+    predict2d_kernel(const __grid_constant__ Predict2DParams P) {
+  __shared__ Pred2Shared<N, T> sh;
+  if (threadIdx.x == 0) {
+    double d = 0.0;
+    sh.go = predictor_step_dt(P.sp, &d, blockIdx.x == 0) ? 1 : 0;
+    sh.dt = d;
+  }
+  __syncthreads();
+  if (!sh.go) return;  // uniform
+  predict2d_block<N, T>(P, sh, sh.dt, nullptr);
 }
 
 // time-integrated rescaled Rusanov flux through the left x-face (dir 0) or the

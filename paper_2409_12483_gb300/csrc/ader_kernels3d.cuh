@@ -113,27 +113,20 @@ struct Pred3Shared {
   int go;
 };
 
-template <int N, int T = 256>
-__global__ void __launch_bounds__(Pred3Cfg<N, T>::THREADS, Pred3Cfg<N, T>::MIN_BLOCKS)
-    predict3d_kernel(const __grid_constant__ Predict3DParams P) {
+// One block of cells in FP64; only: the cells to do (null: all), for the cells that
+// the fixed-point form (ader_fixd.cuh) hands over.
+template <int N, int T>
+__device__ __forceinline__ void predict3d_block(const Predict3DParams& P, Pred3Shared<N, T>& sh,
+                                                double dt, const int* only) {
   using C = Pred3Cfg<N, T>;
   constexpr int n = N + 1, NNN = C::NNN, NST = C::NST, CPB = C::CPB;
-  __shared__ Pred3Shared<N, T> sh;
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    double d = 0.0;
-    sh.go = predictor_step_dt(P.sp, &d, blockIdx.x == 0) ? 1 : 0;
-    sh.dt = d;
-  }
-  __syncthreads();
-  if (!sh.go) return;  // uniform
-  const double dt = sh.dt;
   const double lam[3] = {dt * P.sp.inv_dx, dt * P.inv_dy, dt * P.inv_dz};
   const int lc = tid / NST, node = tid - lc * NST;
   const int p0 = node / NNN, p1 = (node / (n * n)) % n, p2 = (node / n) % n, p3 = node % n;
   const int sp_node = node - p0 * NNN;  // (p1, p2, p3)
   const long long cell = (long long)blockIdx.x * CPB + lc;
-  const bool valid = cell < P.ncells;
+  const bool valid = cell < P.ncells && (!only || only[lc]);
   const OpsD& o = P.ops;
   double uo[kM3], q[kM3];
 #pragma unroll
@@ -166,7 +159,7 @@ __global__ void __launch_bounds__(Pred3Cfg<N, T>::THREADS, Pred3Cfg<N, T>::MIN_B
   const int sc = tid / NNN, sk = tid - sc * NNN;
   const int sd[3] = {sk / (n * n), (sk / n) % n, sk % n};
   const long long scell = (long long)blockIdx.x * CPB + sc;
-  const bool sitem = tid < CPB * NNN && scell < P.ncells;
+  const bool sitem = tid < CPB * NNN && scell < P.ncells && (!only || only[sc]);
   const int cap = P.fixed_iter > 0 ? P.fixed_iter : P.max_iter;
   for (int it = 0; it < cap; ++it) {
     const bool active = !sh.done[lc];
@@ -312,6 +305,20 @@ __global__ void __launch_bounds__(Pred3Cfg<N, T>::THREADS, Pred3Cfg<N, T>::MIN_B
       rec[(6 * NNN + sk) * kM3 + r] = acc;
     }
   }
+}
+
+template <int N, int T = 256>
+__global__ void __launch_bounds__(Pred3Cfg<N, T>::THREADS, Pred3Cfg<N, T>::MIN_BLOCKS)
+    predict3d_kernel(const __grid_constant__ Predict3DParams P) {
+  __shared__ Pred3Shared<N, T> sh;
+  if (threadIdx.x == 0) {
+    double d = 0.0;
+    sh.go = predictor_step_dt(P.sp, &d, blockIdx.x == 0) ? 1 : 0;
+    sh.dt = d;
+  }
+  __syncthreads();
+  if (!sh.go) return;  // uniform
+  predict3d_block<N, T>(P, sh, sh.dt, nullptr);
 }
 
 // The d-direction flux of the 3D Euler equations (the arithmetic of

@@ -161,6 +161,9 @@ struct Predict2DParams {
   double inv_dy;         // 1 / dy (1 / dx travels in sp)
   StepParams sp;
   OpsD ops;
+  OpsI opi;
+  int fix;               // the fixed-point kernel may run (0 < gamma - 1 <= 1)
+  float tolf;
 };
 
 struct Face2DParams {
@@ -198,6 +201,9 @@ struct Predict3DParams {
   double inv_dy, inv_dz;  // 1 / dx travels in sp
   StepParams sp;
   OpsD ops;
+  OpsI opi;
+  int fix;                // the fixed-point kernel may run (0 < gamma - 1 <= 1)
+  float tolf;
 };
 
 struct Face3DParams {
