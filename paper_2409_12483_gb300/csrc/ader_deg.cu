@@ -76,6 +76,14 @@ void launch_update2d_shape(const Face2DParams& p, cudaStream_t s) {
   update2d_kernel<D, T><<<grid_for(p.ncells, U::CPB, 0x7fffffffLL), U::THREADS, 0, s>>>(p);
 }
 
+void launch_update2d(const Face2DParams& p, cudaStream_t s) {
+  if (Upd2Cfg<D, 256>::CPB != Upd2Cfg<D, 128>::CPB &&
+      !use_big_blocks(p.ncells, Upd2Cfg<D, 256>::CPB))
+    launch_update2d_shape<128>(p, s);
+  else
+    launch_update2d_shape<256>(p, s);
+}
+
 // The helpers below are instantiated in every per-degree translation unit with
 // different bodies (they depend on ADER_DEG), so they must have internal linkage.
 // The float-float predictor forms run with a residency target (predict_ff_kernel)
@@ -383,19 +391,27 @@ cudaError_t ADER_CAT(launch_face2d_, ADER_DEG)(const Face2DParams& p, cudaStream
   const long long items = p.ncells * 2 * n;
   const int tpb = flat_threads(items);
   face2d_kernel<D><<<grid_for(items, tpb, 0x7fffffffLL), tpb, 0, s>>>(p);
-  if (Upd2Cfg<D, 256>::CPB != Upd2Cfg<D, 128>::CPB &&
-      !use_big_blocks(p.ncells, Upd2Cfg<D, 256>::CPB))
-    launch_update2d_shape<128>(p, s);
-  else
-    launch_update2d_shape<256>(p, s);
+  launch_update2d(p, s);
   return cudaGetLastError();
 }
 
 cudaError_t ADER_CAT(launch_cfl2d_, ADER_DEG)(const Cfl2DParams& p, cudaStream_t s) {
-  constexpr int Ns = 2 * D + 1;
-  const long long items = p.ncells * Ns * Ns;
-  const int tpb = flat_threads(items);
-  cfl2d_kernel<D><<<grid_for(items, tpb, 0x7fffffffLL), tpb, 0, s>>>(p);
+  // the separable projection of the update kernel in its CFL mode
+  Face2DParams f{};
+  f.u_cfl = p.u;
+  f.cfl_slot = p.slot;
+  f.ncells = p.ncells;
+  f.gamma = p.gamma;
+  f.gm1 = p.gm1;
+  f.inv_dy = p.inv_dy;
+  f.sp.inv_dx = p.inv_dx;
+  f.sp.ctl = p.ctl;
+  for (int j = 0; j < kMaxNs; ++j)
+    for (int k = 0; k < kMaxN; ++k) {
+      f.ops.P[j][k] = p.P[j][k];
+      f.Pf[j][k] = p.Pf[j][k];
+    }
+  launch_update2d(f, s);
   return cudaGetLastError();
 }
 
@@ -522,8 +538,8 @@ cudaError_t ADER_CAT(launch_face_multi_, ADER_DEG)(const FaceParams& p, const Mu
 }
 
 cudaError_t ADER_CAT(launch_cfl_, ADER_DEG)(const CflParams& p, cudaStream_t s) {
-  const long long items = p.dg ? p.ncells * (p.nodal ? D + 1 : p.Ns) : p.ncells;
-  cfl_kernel<D><<<grid_for(items, 256, 152LL * 8), 256, 0, s>>>(p);
+  const long long records = p.dg ? p.ncells * (D + 1) : p.ncells;
+  cfl_kernel<D><<<grid_for(records, kCflCells * (D + 1), 152LL * 6), 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 

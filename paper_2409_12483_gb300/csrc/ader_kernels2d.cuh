@@ -21,9 +21,8 @@
 // update2d_kernel    one thread per (cell, node): volume term minus face terms;
 //                    then the next step's max(lambda_x / dx, lambda_y / dy) over
 //                    the block's cells, projected to the subcells in shared memory.
-// cfl2d_kernel       (the first time step) one thread per (cell, subcell j1, j2): max(lambda_x / dx,
-//                    lambda_y / dy) over the (P (x) P) u subcell averages, an FP32
-//                    screen confirmed in FP64 like the 1D interface kernel's.
+//                    With u_cfl set (the first time step, ader_compute_dt) it only
+//                    takes lambda_max of that state.
 #pragma once
 
 #include "ader_kernels.cuh"  // device helpers, abs_bits, launch parameter structs
@@ -427,15 +426,20 @@ __global__ void __launch_bounds__(Upd2Cfg<N, TB>::THREADS)
   __shared__ float LT[CPB][Ns * Ns];     // FP32 screen: upper bounds of the subcell speeds
   __shared__ float s_cut;
   __shared__ unsigned long long s_wmax[C::THREADS / 32];
-  double dt;
-  int last;
-  if (!corrector_step_dt(P.sp, &dt, &last)) return;  // uniform
+  double dt = 0.0;
+  int last = 0;
+  const bool cfl_only = P.u_cfl != nullptr;  // lambda_max of u_cfl, no update
+  if (!cfl_only && !corrector_step_dt(P.sp, &dt, &last)) return;  // uniform
   const int tid = threadIdx.x;
   const int lc = tid / NN, k = tid - lc * NN;
   const long long cell = (long long)blockIdx.x * CPB + lc;
   const bool valid = tid < C::USED && cell < P.ncells;
   const OpsD& o = P.ops;
-  if (valid) {
+  if (cfl_only) {
+    if (valid)
+#pragma unroll
+      for (int r = 0; r < kM2; ++r) U[lc][k][r] = P.u_cfl[(cell * NN + k) * kM2 + r];
+  } else if (valid) {
     const int k1 = k / n, k2 = k - k1 * n;
     const long long iy = cell / P.nx, ix = cell - iy * P.nx;
     const long long cr = iy * P.nx + (ix + 1 == P.nx ? 0 : ix + 1);
@@ -454,8 +458,8 @@ __global__ void __launch_bounds__(Upd2Cfg<N, TB>::THREADS)
       U[lc][k][r] = un;
     }
   }
-  if (blockIdx.x == 0 && tid == 0) corrector_finish(P.sp, dt, last, true);
-  if (!P.want_lambda) return;  // uniform
+  if (!cfl_only && blockIdx.x == 0 && tid == 0) corrector_finish(P.sp, dt, last, true);
+  if (!cfl_only && !P.want_lambda) return;  // uniform
   __syncthreads();
   // lambda_max of u_new over the Ns^2 subcells, screened as in the 1D interface
   // kernel: the separable projection and bounds on the wave speeds in FP32 for
@@ -538,87 +542,8 @@ __global__ void __launch_bounds__(Upd2Cfg<N, TB>::THREADS)
     }
   }
   const unsigned long long bm = block_max_bits(dbits(lmax), s_wmax);
-  if (tid == 0) atomicMax(&P.sp.ctl->lam[P.sp.par ^ 1], bm);
+  if (tid == 0) atomicMax(&P.sp.ctl->lam[cfl_only ? P.cfl_slot : P.sp.par ^ 1], bm);
   if (bad) atomicOr(&P.sp.ctl->status, kStNonPhysical);
-}
-
-// max over the Ns x Ns subcells of every cell of max(lambda_x / dx, lambda_y / dy)
-// into ctl->lam[slot]; non-physical subcell averages set the status
-template <int N>
-__global__ void __launch_bounds__(256) cfl2d_kernel(const __grid_constant__ Cfl2DParams P) {
-  constexpr int n = N + 1, NN = n * n, Ns = 2 * N + 1;
-  __shared__ unsigned long long s_wmax[8];
-  __shared__ float s_cut;
-  const long long item = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = item < P.ncells * Ns * Ns;
-  long long cell = 0;
-  int j1 = 0, j2 = 0;
-  if (valid) {
-    cell = item / (Ns * Ns);
-    const int j = (int)(item - cell * Ns * Ns);
-    j1 = j / Ns;
-    j2 = j - j1 * Ns;
-  }
-  const double* u = P.u + cell * NN * kM2;
-  const float gf = (float)P.gamma, gm1f = (float)P.gm1;
-  const float ih[2] = {(float)P.inv_dx, (float)P.inv_dy};
-  constexpr float eproj = (float)(2 * n + 6) * 0x1p-24f;  // two FP32 passes
-  float lt = 0.f, lo = 0.f;
-  if (valid) {
-    float v[kM2], e[kM2];
-#pragma unroll
-    for (int r = 0; r < kM2; ++r) {
-      float acc = 0.f, aab = 0.f;
-#pragma unroll
-      for (int k1 = 0; k1 < n; ++k1) {
-        float t = 0.f, at = 0.f;
-#pragma unroll
-        for (int k2 = 0; k2 < n; ++k2) {
-          const float x = d2f_trunc(u[(k1 * n + k2) * kM2 + r]);
-          t = fmaf(P.Pf[j2][k2], x, t);
-          at = fmaf(fabsf(P.Pf[j2][k2]), fabsf(x), at);
-        }
-        acc = fmaf(P.Pf[j1][k1], t, acc);
-        aab = fmaf(fabsf(P.Pf[j1][k1]), at, aab);
-      }
-      v[r] = acc;
-      e[r] = fmaf(eproj, aab, 0x1p-100f);
-    }
-    speed_bounds_f32<2>(v, e, ih, gf, gm1f, lo, lt);
-  }
-  // FP64 below only where the upper bound reaches the block's largest lower bound
-  const unsigned long long fm = block_max_bits((unsigned long long)__float_as_uint(lo), s_wmax);
-  if (threadIdx.x == 0) s_cut = __uint_as_float((unsigned)fm);
-  __syncthreads();
-  double lmax = 0.0;
-  bool bad = false;
-  if (valid && lt >= s_cut) {
-    double v[kM2];
-#pragma unroll
-    for (int r = 0; r < kM2; ++r) {
-      double acc = 0.0;
-#pragma unroll
-      for (int k1 = 0; k1 < n; ++k1) {
-        double t = 0.0;
-#pragma unroll
-        for (int k2 = 0; k2 < n; ++k2) t = fma(P.P[j2][k2], u[(k1 * n + k2) * kM2 + r], t);
-        acc = fma(P.P[j1][k1], t, acc);
-      }
-      v[r] = acc;
-    }
-    const double inv = rcp64(v[0]);
-    const double uu = v[1] * inv, vv = v[2] * inv;
-    const double pp = P.gm1 * fma(neg_half(v[1]), uu, fma(neg_half(v[2]), vv, v[3]));
-    if (!(v[0] > 0.0) || !(pp > 0.0) || !(v[0] < 1.0e300) || !(pp < 1.0e300)) {
-      bad = true;
-    } else {
-      const double c = sqrt64(P.gamma * pp * inv);
-      lmax = fmax((fabs(uu) + c) * P.inv_dx, (fabs(vv) + c) * P.inv_dy);
-    }
-  }
-  const unsigned long long bm = block_max_bits(dbits(lmax), s_wmax);
-  if (threadIdx.x == 0) atomicMax(&P.ctl->lam[P.slot], bm);
-  if (bad) atomicOr(&P.ctl->status, kStNonPhysical);
 }
 
 }  // namespace ader

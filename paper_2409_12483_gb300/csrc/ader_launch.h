@@ -170,6 +170,8 @@ struct Face2DParams {
   const double* trace;
   double* gface;         // [cell][dir][k][4]: fluxes of the left x-face and bottom y-face
   double* u_new;
+  const double* u_cfl;   // non-null: lambda_max of this state only (no update) into lam[cfl_slot]
+  int cfl_slot;
   long long ncells, nx, ny;
   int want_lambda;       // the update also reduces lambda_max of u_new into ctl->lam[par ^ 1]
   double gamma, gm1;
