@@ -28,6 +28,7 @@ struct HostFlags {
   long long steps;
   unsigned long long lam;
   double t;
+  DevCtl ctl;  // the control block at the end of a solve
 };
 
 }  // namespace
@@ -961,7 +962,11 @@ static ader_status solve_impl(ader_ctx* ctx, double* u, double t0, double t_end,
   }
   if ((st = enqueue_cfl(ctx, u, 0)) != ADER_OK) return st;
 
-  const int K = ctx->tune.graph_steps > 0 ? ctx->tune.graph_steps : graph_steps_for(ctx->mesh.n_cells);
+  // steps per graph (even: the state ping-pongs), no more than max_steps needs: a step
+  // after 'done' is a no-op on the device, but its launches are not free (two graphs'
+  // worth of them took 30 % of a 50-step solve on 100 cells)
+  int K = ctx->tune.graph_steps > 0 ? ctx->tune.graph_steps : graph_steps_for(ctx->mesh.n_cells);
+  if (max_steps > 0 && max_steps < K) K = (int)((max_steps + 1) / 2 * 2);
   const bool prof = ctx->opt.profile != 0;
   if (prof && !ctx->pev_ready) {
     for (int j = 0; j < ader_ctx::kMaxGraphSteps; ++j)
@@ -1004,9 +1009,9 @@ static ader_status solve_impl(ader_ctx* ctx, double* u, double t0, double t_end,
     ctx->g_steps = K;
   }
   // Replay K-step graphs; keep two in flight and poll the 'done' flag of the
-  // older one.  Steps after 'done' are no-ops on the device.
-  const long long max_launches =
-      max_steps > 0 ? (max_steps + K - 1) / K + 1 : (long long)4e9 / K;
+  // older one.  Steps after 'done' are no-ops on the device.  max_steps bounds the
+  // graphs: after ceil(max_steps / K) of them the loop is done.
+  const long long max_launches = max_steps > 0 ? (max_steps + K - 1) / K : (long long)4e9 / K;
   long long launches = 0;
   bool finished = false;
   long long steps_seen = 0;
@@ -1045,15 +1050,13 @@ static ader_status solve_impl(ader_ctx* ctx, double* u, double t0, double t_end,
     if (launches >= max_launches) break;
   }
   ctx->launches += launches * (long long)K * kernels_per_step(ctx);
-  CK(cudaMemcpyAsync(&ctx->hflags[0].status, &ctx->ctl->status, sizeof(int),
-                     cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaMemcpyAsync(&ctx->hflags[0].steps, &ctx->ctl->steps, sizeof(long long),
-                     cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaMemcpyAsync(&ctx->hflags[0].t, &ctx->ctl->t, sizeof(double), cudaMemcpyDeviceToHost,
+  const DevCtl& end = ctx->hflags[0].ctl;
+  CK(cudaMemcpyAsync(&ctx->hflags[0].ctl, ctx->ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost,
                      ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
-  const double t_dev = ctx->hflags[0].t;
-  const long long steps = ctx->hflags[0].steps;
+  if (end.done) finished = true;
+  const double t_dev = end.t;
+  const long long steps = end.steps;
   if (steps & 1) {  // the last completed step wrote ubuf
     CK(cudaMemcpyAsync(u, ctx->ubuf, (size_t)state_count(ctx) * sizeof(double),
                        cudaMemcpyDeviceToDevice, ctx->stream));
@@ -1063,7 +1066,7 @@ static ader_status solve_impl(ader_ctx* ctx, double* u, double t0, double t_end,
   if (t_out) *t_out = t_dev;
   if (!finished && !(max_steps > 0 && steps >= max_steps))
     return fail(ctx, ADER_ERR_TIMEOUT, "time loop stopped after %lld graph launches", launches);
-  return status_from_flags(ctx, ctx->hflags[0].status);
+  return status_from_flags(ctx, end.status);
 }
 
 ader_status ader_solve(ader_ctx* ctx, double* u, double t_end, int64_t max_steps,
