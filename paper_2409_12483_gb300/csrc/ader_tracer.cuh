@@ -407,7 +407,9 @@ __global__ void __launch_bounds__(FaceCfg<N, C>::THREADS)
       out[r] = un;
       if (r < kM) {
         sh.base.u[(lc * n + k) * kM + r] = un;
-        sh.base.uf[(lc * n + k) * kM + r] = d2f_trunc(un);
+        const ff uf = d2ff(un);  // both halves: face_lambda's second screen reads them
+        sh.base.uf[(lc * n + k) * kM + r] = uf.hi;
+        sh.base.ufl[(lc * n + k) * kM + r] = uf.lo;
       }
     }
   }
