@@ -10,6 +10,7 @@
 #include "ader_kernels3d.cuh"
 #include "ader_fixd.cuh"
 #include "ader_tracer.cuh"
+#include "ader_fixs.cuh"
 
 #ifndef ADER_DEG
 #error "compile with -DADER_DEG=<0..7>"
@@ -200,6 +201,31 @@ cudaError_t launch_predict_cpb(const PredictParams& p, cudaStream_t s) {
   }
 }
 
+// the nested predictors in fixed point (ader_fixs.cuh)
+template <int SYS>
+cudaError_t launch_fixs(const PredictParams& p, cudaStream_t s) {
+  using C = FixSCfg<D, SYS>;
+  if constexpr (!C::kValid) {
+    return cudaErrorInvalidConfiguration;
+  } else {
+    const long long tiles = (p.ncells + C::CELLS - 1) / C::CELLS;
+    if (tiles <= 0 || tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const long long resident = 152LL * C::MIN_BLOCKS;
+    predict_fixs_kernel<D, SYS><<<(unsigned)(tiles < resident ? tiles : resident), C::THREADS,
+                                  C::kSmemBytes, s>>>(p);
+    return cudaGetLastError();
+  }
+}
+
+template <int SYS>
+cudaError_t prepare_fixs() {
+  using C = FixSCfg<D, SYS>;
+  if constexpr (!C::kValid) return cudaSuccess;
+  else
+    return cudaFuncSetAttribute(predict_fixs_kernel<D, SYS>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes);
+}
+
 // reacting system (ader_source.cuh): predictor tiles of 16 or 32 cells, interface tiles of 32
 template <int CPB>
 cudaError_t prepare_src_cpb() {
@@ -227,6 +253,7 @@ cudaError_t launch_predict_src_cpb(const PredictParams& p, cudaStream_t s) {
 
 cudaError_t launch_predict_src(const PredictParams& p, cudaStream_t s) {
   if (p.prec != 0) return cudaErrorInvalidValue;  // the reacting system runs in FP64
+  if (FixSCfg<D, kSysReacting>::kValid && p.fix && !p.from_q) return launch_fixs<kSysReacting>(p, s);
   // 16-cell tiles wherever the degree allows: the nested loop's per-thread rows
   // in shared memory hold a 32-cell tile to one block per SM (measured at N = 5:
   // 16-cell tiles 7 % faster); the tuned cpb applies to the Euler predictor
@@ -261,6 +288,7 @@ cudaError_t launch_predict_nc_cpb(const PredictParams& p, cudaStream_t s) {
 
 cudaError_t launch_predict_nc(const PredictParams& p, cudaStream_t s) {
   if (p.prec != 0 || p.from_q || p.out_mode != kOutTrace) return cudaErrorInvalidValue;
+  if (FixSCfg<D, kSysTracer>::kValid && p.fix) return launch_fixs<kSysTracer>(p, s);
   // 16-cell tiles wherever the degree allows (as for the reacting system;
   // measured at N = 5: 11 % faster)
   if (NcCfg<D, 16>::kValid) return launch_predict_nc_cpb<16>(p, s);
@@ -310,6 +338,8 @@ cudaError_t ADER_CAT(prepare_degree_, ADER_DEG)() {
     if ((e = prepare_fixd<3, 256>()) != cudaSuccess) return e;
     if ((e = prepare_fixd<3, 64>()) != cudaSuccess) return e;
   }
+  if ((e = prepare_fixs<kSysReacting>()) != cudaSuccess) return e;
+  if ((e = prepare_fixs<kSysTracer>()) != cudaSuccess) return e;
   if ((e = prepare_src_cpb<16>()) != cudaSuccess) return e;
   if ((e = prepare_src_cpb<32>()) != cudaSuccess) return e;
   if constexpr (D <= kMax3DDeg) {  // 3D kernels with more than 48 KB of shared memory

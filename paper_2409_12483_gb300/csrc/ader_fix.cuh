@@ -533,13 +533,11 @@ __device__ __forceinline__ void fix_stage_tables(const PredictParams& P, FixShar
   }
 }
 
-// A block's share of the statistics, then the cells it has to redo (tiles tile0,
-// tile0 + stride, ..).  Every thread of the block.
-template <int N, int WPB>
-__device__ __forceinline__ void fix_finish(const PredictParams& P, const TileIO& io,
-                                           long long tile0, long long stride, double lam,
-                                           double* smem, FixShared<N>& sh, const FixStats& st) {
-  using C = FixCfg<N, WPB>;
+// A block's share of the statistics; whether a cell of the block has to be redone.
+// Every thread of the block.
+template <int N>
+__device__ __forceinline__ bool fix_block_stats(const TileIO& io, FixShared<N>& sh,
+                                                const FixStats& st) {
   const int itmax = __reduce_max_sync(0xffffffffu, st.itmax);
   const int itsum = __reduce_add_sync(0xffffffffu, st.itsum);
   const int ncells = __reduce_add_sync(0xffffffffu, st.ncells);
@@ -558,7 +556,16 @@ __device__ __forceinline__ void fix_finish(const PredictParams& P, const TileIO&
     atomicAdd((unsigned long long*)&c->iter_cells, (unsigned long long)sh.ncells);
     if (sh.bad) atomicOr(&c->status, kStNotConverged);
   }
-  if (redo) {
+  return redo;
+}
+
+// The same, then the cells to redo (tiles tile0, tile0 + stride, ..).
+template <int N, int WPB>
+__device__ __forceinline__ void fix_finish(const PredictParams& P, const TileIO& io,
+                                           long long tile0, long long stride, double lam,
+                                           double* smem, FixShared<N>& sh, const FixStats& st) {
+  using C = FixCfg<N, WPB>;
+  if (fix_block_stats<N>(io, sh, st)) {
     const long long tiles = (io.ncells + C::CELLS - 1) / C::CELLS;
     for (long long t = tile0; t < tiles; t += stride) {
       fix_redo<N, WPB>(P, io, t, lam, smem, sh.redo);

@@ -129,14 +129,15 @@ constexpr int kFxSV[8] = {0, 2, 3, 4, 5, 5, 5, 6};
 // The Euler fluxes of D directions in fixed point: q = (rho, m_1 .. m_D, E), rho and m
 // at frac 61, E at frac 57, all below 2 in magnitude, to F[d] = (m_d, m_j u_d + p
 // (j = d), (E + p) u_d) at frac 57.  g2h, g2l: (gamma - 1) / 2 <= 1/2 at frac 62.  `bad`
-// collects nonzero bits when rho is not above 1/8, a |u_d| leaves 2 or a flux leaves 8.
+// collects nonzero bits when rho is not above 1/8, a |u_d| leaves 2 or a flux leaves 8;
+// velocity: the u_d as limbs at frac 60.
 //   r   = 1 / rho to 2^-28: float reciprocal of the high limb, one Newton step;
 //   u   = u0 + (m - rho u0) r, u0 = m r at frac 28: the remainder is below 2^-26 and
 //         exact to 2^-57, so 32-bit arithmetic modulo 2^32 gives it at frac 57;
 //   the products' l l terms, left out, stay below 2^-56 (rms 2^-57).
 template <int D>
 ADER_HD void fx_fluxes(const fxi (&q)[D + 2], int g2h, int g2l, fxi (&F)[D][D + 2],
-                       unsigned& bad) {
+                       unsigned& bad, Fx2* velocity = nullptr) {
   const Fx2 R = fx_split(q[0]);
   bad |= (unsigned)(R.h - 0x4100000) & 0x80000000u;
 #ifdef __CUDA_ARCH__
@@ -169,6 +170,7 @@ ADER_HD void fx_fluxes(const fxi (&q)[D + 2], int g2h, int g2l, fxi (&F)[D][D + 
     U[d] = fx_split(fx_join((unsigned)(fx_hi(us) >> 25),
                             fx_funnel_l((unsigned)fx_lo(us), (unsigned)fx_hi(us), 7)));
     U[d].h = (int)((unsigned)U[d].h + (unsigned)u0);  // u0 + (us >> 25) at frac 60
+    if (velocity) velocity[d] = U[d];
 #ifdef __CUDACC__
 #pragma unroll
 #endif

@@ -100,11 +100,12 @@ __device__ __forceinline__ bool block_step_dt_src(const StepParams& sp, double* 
   return go;
 }
 
-template <int N, int CPB>
+// CELLS, THREADS and `only` as in predict_tile (the fixed-point form's leftovers)
+template <int N, int CPB, int CELLS = CPB, int THREADS = SrcCfg<N, CPB>::THREADS>
 __device__ __forceinline__ void predict_src_tile(const PredictParams& P, const TileIO& io,
                                                  long long tile, double dt, double* smem,
-                                                 SrcShared<N>& sh) {
-  constexpr int n = N + 1, M = kMR, THREADS = SrcCfg<N, CPB>::THREADS, RS = n * M;
+                                                 SrcShared<N>& sh, const int* only = nullptr) {
+  constexpr int n = N + 1, M = kMR, RS = n * M;
   const double lam = dt * P.sp.inv_dx;
   double* sd = smem;                   // exchange rows
   double* sg = sd + CPB * n * RS;      // frozen (dt/dx) k~ F rows (own row per thread)
@@ -113,8 +114,8 @@ __device__ __forceinline__ void predict_src_tile(const PredictParams& P, const T
 
   const int tid = threadIdx.x;
   const int lc = tid / n, p0 = tid - lc * n;
-  const long long cell = tile * CPB + lc;
-  const bool valid = cell < io.ncells;
+  const long long cell = tile * CELLS + lc;
+  const bool valid = (CELLS == CPB || lc < CELLS) && cell < io.ncells && (!only || only[lc]);
   for (int i = tid; i < 2 * kMaxCpb * 2; i += THREADS) (&sh.red[0][0][0])[i] = 0ull;
   for (int i = tid; i < kMaxCpb * 2; i += THREADS) (&sh.ored[0][0])[i] = 0ull;
   if (tid == 0) {

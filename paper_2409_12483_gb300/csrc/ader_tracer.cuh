@@ -77,11 +77,12 @@ __device__ __forceinline__ void nc_row_b(const double (&q)[N + 1][kMN], const Op
   }
 }
 
-template <int N, int CPB>
+// CELLS, THREADS and `only` as in predict_tile (the fixed-point form's leftovers)
+template <int N, int CPB, int CELLS = CPB, int THREADS = NcCfg<N, CPB>::THREADS>
 __device__ __forceinline__ void predict_nc_tile(const PredictParams& P, const TileIO& io,
                                                 long long tile, double dt, double* smem,
-                                                SrcShared<N>& sh) {
-  constexpr int n = N + 1, M = kMN, THREADS = NcCfg<N, CPB>::THREADS, RS = n * M;
+                                                SrcShared<N>& sh, const int* only = nullptr) {
+  constexpr int n = N + 1, M = kMN, RS = n * M;
   const double lam = dt * P.sp.inv_dx;
   double* sd = smem;                   // exchange rows
   double* sg = sd + CPB * n * RS;      // frozen (dt/dx) k~ F rows (own row per thread)
@@ -90,8 +91,8 @@ __device__ __forceinline__ void predict_nc_tile(const PredictParams& P, const Ti
 
   const int tid = threadIdx.x;
   const int lc = tid / n, p0 = tid - lc * n;
-  const long long cell = tile * CPB + lc;
-  const bool valid = cell < io.ncells;
+  const long long cell = tile * CELLS + lc;
+  const bool valid = (CELLS == CPB || lc < CELLS) && cell < io.ncells && (!only || only[lc]);
   for (int i = tid; i < 2 * kMaxCpb * 2; i += THREADS) (&sh.red[0][0][0])[i] = 0ull;
   for (int i = tid; i < kMaxCpb * 2; i += THREADS) (&sh.ored[0][0])[i] = 0ull;
   if (tid == 0) {
