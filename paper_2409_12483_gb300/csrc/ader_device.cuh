@@ -302,6 +302,23 @@ __device__ __forceinline__ void speed_bounds_f32(const float (&v)[D + 2], const 
   hi = l_hi;
 }
 
+// The cut of the lambda_max screens.  lo: the largest FP32 lower bound of a block's
+// speeds.  It is published in the slot of lambda_max itself, where it can do no
+// harm: the subcell it belongs to has an FP64 speed of at least lo, and the subcell
+// with the largest speed is above every cut, so it is always evaluated.  What the
+// slot held before, other blocks' bounds and maxima, is a cut too (rounded down):
+// on a mesh whose speeds vary, most blocks then have nothing left for FP64 (a warp's
+// FP64 instruction takes 64 cycles of its scheduler, a candidate ~60 of them).
+// Interface kernel N = 5, 10^5 cells 76 -> 63 us, N = 7, 10^6 cells 750 -> 577 us; 2D
+// update N = 5, 160 x 157 cells 170 -> 115 us.
+__device__ __forceinline__ float lambda_cut(unsigned long long* lam, float lo) {
+  const unsigned b = __float_as_uint(lo);  // exact as a double, zero and subnormals as 0
+  const unsigned long long d =
+      (b >> 23) ? ((unsigned long long)((b >> 23) + 896u) << 52) | ((unsigned long long)(b & 0x7fffffu) << 29)
+                : 0ull;
+  return fmaxf(lo, d2f_trunc(bitsd(atomicMax(lam, d))));
+}
+
 // x > 0 and finite, tested on the bit pattern (integer pipe, no FP64 compare)
 __device__ __forceinline__ bool pos_finite(double x) {
   return dbits(x) - 1ull < 0x7fefffffffffffffull;

@@ -1029,9 +1029,12 @@ __device__ __forceinline__ void face_lambda(const FaceParams& P, const StepParam
     lo_loc = fmaxf(lo_loc, lo);
   }
   unsigned long long fm = block_max_bits((unsigned long long)__float_as_uint(lo_loc), sh.wmax);
-  if (tid == 0) sh.lt_cut = __uint_as_float((unsigned)fm);
+  if (tid == 0) sh.lt_cut = lambda_cut(&sp.ctl->lam[sp.par ^ 1], __uint_as_float((unsigned)fm));
   __syncthreads();
   const float cut = sh.lt_cut;
+  bool any = false;
+  for (int item = tid; item < items; item += THREADS) any |= sh.lt[item] >= cut;
+  if (!__syncthreads_or(any)) return;  // another tile holds the maximum
   // (2) the float-float screen; per-subcell upper bounds (ff_key; 0 marks a
   // subcell left out by (1)) go to the flux array, free since the update
   unsigned long long* hi2 = reinterpret_cast<unsigned long long*>(sh.G);
@@ -1304,10 +1307,8 @@ __global__ void __launch_bounds__(FaceCfg<N, C>::THREADS)
 // every subcell costs 6 n + 15 operations on a pipe of 2 lanes per SM (DG N = 5,
 // 10^5 cells 92 us; N = 7, 10^6 cells 1.0 ms).  Here FP32 bounds on every speed
 // (speed_bounds_f32, as in face_lambda) leave to FP64 the subcells whose upper
-// bound reaches the largest lower bound the block knows: its own so far, or any
-// block's published maximum.  Every value used as that cut is a lower bound of
-// lambda_max, so the maximum is the FP64 one.  A DG N = 7 step on 10^6 cells with the
-// CFL time step went from 4.28 to 3.32 ms.
+// bound reaches the cut of lambda_cut (N = 5, 10^5 cells 22 us; N = 7, 10^6 cells 175 us;
+// with a cut per warp and tile only, the first round's candidates alone took 36 us).
 // Items are subcells (cell, j) of a 64-cell tile, its state as floats in shared
 // memory; for FV the cells, for cfl_mode 1 the nodes.
 constexpr int kCflCells = 64;
@@ -1316,15 +1317,16 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflPar
   constexpr int n = N + 1, Ns = 2 * N + 1, T = 256;
   __shared__ unsigned long long s_wmax[32];
   __shared__ float uf[kCflCells * n * kM];
+  __shared__ float lt[kCflCells * Ns];  // upper bounds (n <= Ns)
   __shared__ float Pf[Ns * n];
-  __shared__ unsigned s_cut;
+  __shared__ float s_cut;
   const int tid = threadIdx.x;
   const bool proj = P.dg && !P.nodal;
   const float gf = (float)P.gamma, gm1f = (float)P.gm1;
   const float one[1] = {1.f};
   const float eproj = proj ? (float)(n + 4) * 0x1p-24f : 0x1p-22f;
+  unsigned long long* lam = &P.ctl->lam[P.slot];
   for (int i = tid; i < Ns * n; i += T) Pf[i] = (float)P.ops.P[i / n][i % n];
-  if (tid == 0) s_cut = 0u;
   double lmax = 0.0;
   bool bad = false;
   // records of P.vars values, the Euler variables (rho, m, E) first: DG nodes, FV cells
@@ -1338,64 +1340,60 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflPar
       const int k = i / kM, r = i - k * kM;
       uf[i] = d2f_trunc(u0[k * P.vars + r]);
     }
-    // any block's maximum so far, rounded down
-    if (tid == 0)
-      atomicMax(&s_cut, __float_as_uint(d2f_trunc(
-                            bitsd(*(volatile unsigned long long*)&P.ctl->lam[P.slot]))));
     __syncthreads();
     const int items = proj ? nrec / n * Ns : nrec;
-    for (int i0 = 0; i0 < items; i0 += T) {
-      const int item = i0 + tid;
-      const int lc = proj ? item / Ns : item, j = proj ? item - lc * Ns : 0;
-      float lo = 0.f, hi = -1.f;
-      if (item < items) {
-        float v[kM], e[kM];
-        if (proj) {
-#pragma unroll
-          for (int r = 0; r < kM; ++r) {
-            float acc = 0.f, aab = 0.f;
-#pragma unroll
-            for (int k = 0; k < n; ++k) {
-              const float pk = Pf[j * n + k], x = uf[(lc * n + k) * kM + r];
-              acc = fmaf(pk, x, acc);
-              aab = fmaf(fabsf(pk), fabsf(x), aab);
-            }
-            v[r] = acc;
-            e[r] = fmaf(eproj, aab, 0x1p-100f);
-          }
-        } else {
-#pragma unroll
-          for (int r = 0; r < kM; ++r) {
-            v[r] = uf[item * kM + r];
-            e[r] = fmaf(eproj, fabsf(v[r]), 0x1p-100f);
-          }
-        }
-        speed_bounds_f32<1>(v, e, one, gf, gm1f, lo, hi);
-      }
-      const unsigned wlo = __reduce_max_sync(0xffffffffu, __float_as_uint(lo));
-      if ((tid & 31) == 0) atomicMax(&s_cut, wlo);
-      __syncwarp();
-      if (hi >= __uint_as_float(*(volatile unsigned*)&s_cut)) {
-        double v[kM];
+    float lo_loc = 0.f;
+    for (int item = tid; item < items; item += T) {
+      float v[kM], e[kM], lo;
+      if (proj) {
+        const int lc = item / Ns, j = item - lc * Ns;
 #pragma unroll
         for (int r = 0; r < kM; ++r) {
-          double acc = 0.0;
-          if (proj) {
+          float acc = 0.f, aab = 0.f;
 #pragma unroll
-            for (int k = 0; k < n; ++k)
-              acc = fma(P.ops.P[j][k], u0[(long long)(lc * n + k) * P.vars + r], acc);
-          } else {
-            acc = u0[(long long)item * P.vars + r];
+          for (int k = 0; k < n; ++k) {
+            const float pk = Pf[j * n + k], x = uf[(lc * n + k) * kM + r];
+            acc = fmaf(pk, x, acc);
+            aab = fmaf(fabsf(pk), fabsf(x), aab);
           }
           v[r] = acc;
+          e[r] = fmaf(eproj, aab, 0x1p-100f);
         }
-        lmax = fmax(lmax, wave_speed(v, P.gamma, P.gm1, &bad));
+      } else {
+#pragma unroll
+        for (int r = 0; r < kM; ++r) {
+          v[r] = uf[item * kM + r];
+          e[r] = fmaf(eproj, fabsf(v[r]), 0x1p-100f);
+        }
       }
+      speed_bounds_f32<1>(v, e, one, gf, gm1f, lo, lt[item]);
+      lo_loc = fmaxf(lo_loc, lo);
     }
-    // publish the tile's maximum for the other blocks' cuts
-    const unsigned long long bm = block_max_bits(dbits(lmax), s_wmax);
-    if (tid == 0 && bm) atomicMax(&P.ctl->lam[P.slot], bm);
+    const unsigned long long fm = block_max_bits((unsigned long long)__float_as_uint(lo_loc), s_wmax);
+    if (tid == 0) s_cut = lambda_cut(lam, __uint_as_float((unsigned)fm));
+    __syncthreads();
+    const float cut = s_cut;
+    for (int item = tid; item < items; item += T) {
+      if (!(lt[item] >= cut)) continue;
+      const int lc = proj ? item / Ns : item, j = proj ? item - lc * Ns : 0;
+      double v[kM];
+#pragma unroll
+      for (int r = 0; r < kM; ++r) {
+        double acc = 0.0;
+        if (proj) {
+#pragma unroll
+          for (int k = 0; k < n; ++k)
+            acc = fma(P.ops.P[j][k], u0[(long long)(lc * n + k) * P.vars + r], acc);
+        } else {
+          acc = u0[(long long)item * P.vars + r];
+        }
+        v[r] = acc;
+      }
+      lmax = fmax(lmax, wave_speed(v, P.gamma, P.gm1, &bad));
+    }
   }
+  const unsigned long long bm = block_max_bits(dbits(lmax), s_wmax);
+  if (tid == 0 && bm) atomicMax(lam, bm);
   if (bad) atomicOr(&P.ctl->status, kStNonPhysical);
 }
 

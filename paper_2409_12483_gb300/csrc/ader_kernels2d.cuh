@@ -509,7 +509,9 @@ __global__ void __launch_bounds__(Upd2Cfg<N, TB>::THREADS)
     lo_loc = fmaxf(lo_loc, lo);
   }
   const unsigned long long fm = block_max_bits((unsigned long long)__float_as_uint(lo_loc), s_wmax);
-  if (tid == 0) s_cut = __uint_as_float((unsigned)fm);
+  if (tid == 0)
+    s_cut = lambda_cut(&P.sp.ctl->lam[cfl_only ? P.cfl_slot : P.sp.par ^ 1],
+                       __uint_as_float((unsigned)fm));
   __syncthreads();
   const float cut = s_cut;
   double lmax = 0.0;

@@ -1065,7 +1065,9 @@ __global__ void __launch_bounds__(Upd3Cfg<N, TB>::THREADS)
     lo_loc = fmaxf(lo_loc, lo);
   }
   const unsigned long long fm = block_max_bits((unsigned long long)__float_as_uint(lo_loc), s_wmax);
-  if (tid == 0) s_cut = __uint_as_float((unsigned)fm);
+  if (tid == 0)
+    s_cut = lambda_cut(&P.sp.ctl->lam[cfl_only ? P.cfl_slot : P.sp.par ^ 1],
+                       __uint_as_float((unsigned)fm));
   __syncthreads();
   const float cut = s_cut;
   double lmax = 0.0;
@@ -1167,7 +1169,7 @@ __global__ void __launch_bounds__(256) cfl3d_kernel(const __grid_constant__ Cfl3
   }
   // FP64 below only where the upper bound reaches the block's largest lower bound
   const unsigned long long fm = block_max_bits((unsigned long long)__float_as_uint(lo), s_wmax);
-  if (threadIdx.x == 0) s_cut = __uint_as_float((unsigned)fm);
+  if (threadIdx.x == 0) s_cut = lambda_cut(&P.ctl->lam[P.slot], __uint_as_float((unsigned)fm));
   __syncthreads();
   double lmax = 0.0;
   bool bad = false;

@@ -615,7 +615,8 @@ __global__ void __launch_bounds__(128) lim_finish_kernel(const __grid_constant__
     if (own) lo_loc = fmaxf(lo_loc, lo);
   }
   const unsigned long long fm = block_max_bits((unsigned long long)__float_as_uint(lo_loc), s_wmax);
-  if (threadIdx.x == 0) s_cut = __uint_as_float((unsigned)fm);
+  if (threadIdx.x == 0)
+    s_cut = lambda_cut(&P.sp.ctl->lam[P.sp.par ^ 1], __uint_as_float((unsigned)fm));
   __syncthreads();
   const float cut = s_cut;
   // The subcells left to FP64 are few and spread thinly over the cells (on a
