@@ -206,6 +206,7 @@ FaceParams make_face(const ader_ctx* c, const double* v_old, double* u_new, cons
   f.nodal = c->opt.cfl_mode == 1;
   f.gamma = c->opt.gamma;
   f.gm1 = c->opt.gamma - 1.0;
+  f.gas = make_fx_gas(f.gamma);
   f.sp = sp;
   f.ops = c->basis.d;
   return f;
@@ -366,6 +367,7 @@ ader_status enqueue_step2d(ader_ctx* ctx, const double* src, double* dst, const 
   f.ny = ctx->ny;
   f.gamma = ctx->opt.gamma;
   f.gm1 = ctx->opt.gamma - 1.0;
+  f.gas = make_fx_gas(f.gamma);
   f.inv_dy = 1.0 / ctx->dy;
   f.want_lambda = want_lambda;  // the predictor of this step has reset the slot
   f.sp = sp;
@@ -411,6 +413,7 @@ ader_status enqueue_step3d(ader_ctx* ctx, const double* src, double* dst, const 
   f.nz = ctx->nz;
   f.gamma = ctx->opt.gamma;
   f.gm1 = ctx->opt.gamma - 1.0;
+  f.gas = make_fx_gas(f.gamma);
   f.inv_dy = 1.0 / ctx->dy;
   f.inv_dz = 1.0 / ctx->dz;
   f.want_lambda = want_lambda;  // the predictor of this step has reset the slot

@@ -32,6 +32,7 @@
 
 #include "ader_device.cuh"
 #include "ader_ff.cuh"
+#include "ader_fixr.cuh"
 #include "ader_launch.h"
 
 namespace ader {
@@ -1183,7 +1184,8 @@ __device__ __forceinline__ void face_tile(const FaceParams& P, const FaceIO& io,
         g[r] = m;
       }
     }
-    rusanov2_screened(a, b, G2, P.gamma, P.gm1, (float)P.gamma);
+    if (!fx_rusanov2<1, 0>(a, b, G2, P.gas))
+      rusanov2_screened(a, b, G2, P.gamma, P.gm1, (float)P.gamma);
 #pragma unroll
     for (int r = 0; r < kM; ++r) sh.G[(f * n + l0) * kM + r] = G2[r];
   }
@@ -1261,23 +1263,13 @@ __device__ __forceinline__ void face_update_block(const FaceParams& P, FaceShare
   corrector_finish(P.sp, dt, last, blockIdx.x == 0 && threadIdx.x == 0);
 }
 
+// 4 resident blocks (64 registers): the fixed-point flux alone would take 71-74 (3
+// blocks), and the short phases between barriers want warps to fill them.  3 / 4 / 5
+// blocks: N = 3, 1e5 cells 45.4 / 41.9 / 45.6 us, N = 4, 1e6 cells 387 / 358 / 380,
+// N = 5, 1e5 cells 50.9 / 47.6 / 54.4, N = 7, 1e6 cells 485 / 426 / 450.
 template <int N, int C = 64>
-__global__ void __launch_bounds__(FaceCfg<N, C>::THREADS)
+__global__ void __launch_bounds__(FaceCfg<N, C>::THREADS, 4)
     face_update_kernel(const __grid_constant__ FaceParams P) {
-  __shared__ FaceShared<N, C> sh;
-  face_update_block<N, C>(P, sh);
-}
-
-// The same kernel with 5 resident blocks asked of the register allocation.  The
-// compiler's choice (56-70 registers) leaves 4 blocks from N = 5, and the
-// kernel's short phases between barriers are latency-bound there: 5 blocks
-// (48 registers) measured 7-15 % faster at N = 5 and 7 on 10^6 cells and the
-// same at N = 5 on 10^5.  Below N = 5 (48 registers, 5 blocks already) naming
-// a block count only made the allocation worse, so those degrees keep
-// face_update_kernel.
-template <int N, int C = 64>
-__global__ void __launch_bounds__(FaceCfg<N, C>::THREADS, 5)
-    face_update_occ_kernel(const __grid_constant__ FaceParams P) {
   __shared__ FaceShared<N, C> sh;
   face_update_block<N, C>(P, sh);
 }

@@ -58,6 +58,7 @@ struct FaceParams {
   int Ns;
   int nodal;             // DG: lambda_max over the nodal values (cfl_mode 1), not the subcells
   double gamma, gm1;
+  FxGas gas;
   StepParams sp;
   OpsD ops;
 };
@@ -175,6 +176,7 @@ struct Face2DParams {
   long long ncells, nx, ny;
   int want_lambda;       // the update also reduces lambda_max of u_new into ctl->lam[par ^ 1]
   double gamma, gm1;
+  FxGas gas;
   double inv_dy;
   StepParams sp;
   OpsD ops;
@@ -217,6 +219,7 @@ struct Face3DParams {
   long long ncells, nx, ny, nz;
   int want_lambda;       // the update also reduces lambda_max of u_new into ctl->lam[par ^ 1]
   double gamma, gm1;
+  FxGas gas;
   double inv_dy, inv_dz;
   StepParams sp;
   OpsD ops;

@@ -170,6 +170,21 @@ bool set_fx_gamma(double gamma, OpsI* o) {
   return true;
 }
 
+FxGas make_fx_gas(double gamma) {
+  FxGas g{};
+  OpsI o;
+  g.ok = set_fx_gamma(gamma, &o) ? 1 : 0;
+  if (!g.ok) return g;
+  g.g2h = o.g2[0];
+  g.g2l = o.g2[1];
+  int h[2];
+  split_fx((ld)gamma, 60, h);
+  g.gh = h[0];
+  g.gl = h[1];
+  g.gammaf = (float)gamma;
+  return g;
+}
+
 int build_basis(int N, bool weno, Basis* out) {
   if (!out || N < 0 || N > kMaxDeg) return -1;
   std::memset(out, 0, sizeof(*out));

@@ -102,6 +102,16 @@ void split_fx(long double x, int frac, int out[2]);
 // (gamma - 1) / 2 at frac 62; false when the fixed-point form cannot hold it.
 bool set_fx_gamma(double gamma, OpsI* o);
 
+// gamma and (gamma - 1) / 2 of an interface kernel; ok: the fixed-point form may run
+struct FxGas {
+  int g2h, g2l;  // (gamma - 1) / 2 at frac 62
+  int gh, gl;    // gamma at frac 60
+  float gammaf;
+  int ok;
+};
+// the same and gamma itself, for the interface kernels (ader_fixr.cuh)
+FxGas make_fx_gas(double gamma);
+
 // Returns 0 on success.  weno != 0 also builds the WENO tables (N even, 2 <= N).
 int build_basis(int N, bool weno, Basis* out);
 

@@ -190,6 +190,7 @@ FaceParams server_face_params(const ader_server* srv, int N) {
   f.Ns = srv->basis[N].Ns;
   f.gamma = srv->opt.gamma;
   f.gm1 = srv->opt.gamma - 1.0;
+  f.gas = make_fx_gas(f.gamma);
   f.ops = srv->basis[N].d;
   return f;
 }
