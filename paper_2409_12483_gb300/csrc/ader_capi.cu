@@ -63,11 +63,10 @@ struct ader_ctx {
   // [shard_first, shard_first + shard_local) held at offset shard_halo
   long long shard_first = -1, shard_local = 0, shard_global = 0;
   int shard_halo = 0;
-  float* lim_mmf = nullptr;   // limiter: FP32 subcell extrema of u^n and bounds [cell][9]
   Sub1Ops sub1{};             // limiter: degree-1 operators of the subcell scheme
   int* lim_flag = nullptr;    // limiter: troubled flags [cell]
-  long long* lim_list = nullptr;  // limiter: troubled-cell list [cell]
-  double* lim_gface = nullptr;    // limiter: subcell fluxes of troubled cells' faces [cell][6]
+  long long* lim_list = nullptr;  // limiter: list of cells to recompute [cell]
+  double* lim_gface = nullptr;    // limiter: flux corrections of troubled cells' faces [cell][6]
   // cached solve graph
   cudaGraphExec_t gexec = nullptr;
   const double* g_u = nullptr;
@@ -128,8 +127,7 @@ size_t workspace_bytes(const ader_ctx* c) {
   if (c->dims == 2) b += align_up((size_t)c->mesh.n_cells * 2 * c->n * kM2 * sizeof(double));
   if (c->dims == 3) b += align_up((size_t)c->mesh.n_cells * 3 * c->n * c->n * kM3 * sizeof(double));
   if (c->opt.limiter)
-    b += align_up((size_t)c->mesh.n_cells * 9 * sizeof(float)) +
-         align_up((size_t)c->mesh.n_cells * 6 * sizeof(double)) +
+    b += align_up((size_t)c->mesh.n_cells * 6 * sizeof(double)) +
          align_up((size_t)c->mesh.n_cells * sizeof(long long)) +
          align_up((size_t)c->mesh.n_cells * sizeof(int));
   return b;
@@ -138,7 +136,7 @@ size_t workspace_bytes(const ader_ctx* c) {
 int kernels_per_step(const ader_ctx* c) {
   if (c->dims >= 2) return 3;  // predictor, face fluxes, update with lambda_max
   int k = c->scheme == ADER_SCHEME_WENO_FV ? 3 : 2;
-  if (c->opt.limiter) k += 4;
+  if (c->opt.limiter) k += 3;
   return k;
 }
 
@@ -299,7 +297,6 @@ ader_status enqueue_limiter(ader_ctx* ctx, const double* src, double* dst, const
   l.u_old = src;
   l.u = dst;
   l.trace = ctx->trace;
-  l.mmf = ctx->lim_mmf;
   l.troubled = ctx->lim_flag;
   l.list = ctx->lim_list;
   l.gface = ctx->lim_gface;
@@ -330,7 +327,7 @@ ader_status enqueue_limiter(ader_ctx* ctx, const double* src, double* dst, const
   }
   l.pabs = (float)(pabs * (1.0 + 1e-6));  // rounded up
   CK(do_limiter(ctx->N, l, ctx->stream));
-  ctx->launches += 4;
+  ctx->launches += 3;
   return ADER_OK;
 }
 
@@ -815,8 +812,6 @@ ader_status ader_bind(ader_ctx* ctx, void* ws, size_t bytes, void* stream) {
     p += align_up((size_t)ctx->mesh.n_cells * 3 * ctx->n * ctx->n * kM3 * sizeof(double));
   }
   if (ctx->opt.limiter) {
-    ctx->lim_mmf = reinterpret_cast<float*>(p);
-    p += align_up((size_t)ctx->mesh.n_cells * 9 * sizeof(float));
     ctx->lim_gface = reinterpret_cast<double*>(p);
     p += align_up((size_t)ctx->mesh.n_cells * 6 * sizeof(double));
     ctx->lim_list = reinterpret_cast<long long*>(p);

@@ -32,7 +32,7 @@ struct DevCtl {
   int iter_max;
   int pad_;
   unsigned long long troubled;  // cells marked by the limiter's detectors (summed over steps)
-  unsigned long long lim_n;     // entries of the limiter's troubled-cell list (this step)
+  unsigned long long lim_n;     // entries of the limiter's cell list (zero between steps)
 };
 
 // How a launch gets its time step.

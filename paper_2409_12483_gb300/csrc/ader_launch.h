@@ -129,11 +129,11 @@ struct LimParams {
   const double* u_old;   // u^n, [cell][n][3]
   double* u;             // in: candidate u*, out: u^{n+1} (same layout)
   const double* trace;   // predictor traces [cell][qR(3n) | qL(3n) | u + volume(3n)]
-  float* mmf;            // [cell][9]: FP32 min (3), max (3) of the subcell averages of
-                         // u^n and a bound (3) on their distance from the FP64 ones
   int* troubled;         // [cell]
-  long long* list;       // [cell]: the troubled cells of the step (first ctl->lim_n entries)
-  double* gface;         // [cell][2][3]: subcell fluxes of a troubled cell's left / right face
+  long long* list;       // [cell]: cells of the step to recompute (first ctl->lim_n entries);
+                         // ~cell: left to the FP64 detectors
+  double* gface;         // [cell][2][3]: subcell flux minus DG flux of a troubled cell's
+                         // left / right face
   long long ncells;
   int bc;                // kBcPeriodic or kBcOutflow
   int Ns;

@@ -5,36 +5,41 @@
 // limiter of Sec. 2).  Run after the interface kernel has written the candidate
 // u* in place of u^{n+1}:
 //
-// lim_minmax_kernel  per cell, the 2N+1 subcell averages P u^n in FP32: their
-//                    minimum and maximum per variable and a bound on their
-//                    distance from the FP64 averages.
 // lim_detect_kernel  per cell, PAD (rho > 0, e > 0) on the subcell averages P u*
 //                    and the relaxed discrete maximum principle against the
-//                    extrema of the cell and its neighbours, delta = max(delta0,
-//                    eps (max - min)); marks troubled cells (mode 2: every cell),
-//                    counts them.  An FP32 pass clears the cells that pass with
-//                    the error bounds to spare; the rest are decided in FP64,
-//                    so every flag is the FP64 detectors' flag.
-// lim_recompute_kernel  one half-warp per listed troubled cell: the ADER-WENO2
-//                    scheme on its 2N+1 subcells from P u^n (item j: degree-1
-//                    WENO and the degree-1 LST-DG predictor of subcell j - 1,
-//                    the neighbours' boundary subcells included; item f: the
-//                    Rusanov flux through subcell face f averaged over the two
-//                    tau nodes; items spread over the group's 16 lanes), the subcell update, the pseudo-inverse
-//                    reconstruction R = (P^T P)^-1 P^T with the mean of the
-//                    subcell values as fallback when R v has an inadmissible
-//                    subcell average; the fluxes of the cell's own faces go to
-//                    gface for the neighbours.
+//                    extrema of P u^n over the cell and its neighbours, delta =
+//                    max(delta0, eps (max - min)), in FP32 with error bounds
+//                    (mode 2: every cell is troubled).  Cells that pass with the
+//                    bounds to spare are cleared; the others are listed.
+// lim_recompute_kernel  one block per listed cell, its lanes sharing the work of
+//                    each phase: the FP64 detectors (so every flag is the FP64
+//                    detectors' flag), then, where the cell is troubled, the
+//                    ADER-WENO2 scheme on its 2N+1 subcells from P u^n (degree-1
+//                    WENO and LST-DG predictor of every subcell, the neighbours'
+//                    boundary subcells included; the Rusanov flux through each
+//                    subcell face averaged over the two tau nodes), the subcell
+//                    update, the pseudo-inverse reconstruction R = (P^T P)^-1 P^T
+//                    with the mean of the subcell values as fallback when R v has
+//                    an inadmissible subcell average; and, for the neighbours, the
+//                    difference between the subcell flux and the DG flux (from the
+//                    predictor traces) of the cell's own two faces.
 // lim_finish_kernel  per cell: a DG cell next to a troubled one has its update
-//                    corrected by the difference between the subcell flux and
-//                    its DG flux (recomputed from the predictor traces) on the
-//                    shared face, so the step stays conservative; then the
+//                    corrected by that difference on the shared face, so the step
+//                    stays conservative; then the
 //                    screened lambda_max of the limited state for the next
 //                    step (the CFL reduction of the unlimited path's interface
 //                    kernel, moved here because the limiter changes the state).
 //
-// The detectors run one thread per cell; the recomputation touches only the
-// listed cells.  Both cells of a face between two troubled cells form its flux
+// What bounds it.  A few listed cells per step: the chains of dependent FP64
+// instructions of lone warps (64 cycles each), not bandwidth.  So nothing in FP64 is
+// left to one lane that several can share: detectors by (neighbour, subcell,
+// variable), predictor by (subcell, space-time node), fluxes by (face, tau node).
+// Sod tube, N = 3, 10007 cells, per step, against one lane per cell in the detectors and
+// per subcell in the recomputation: detectors 40 -> 10 us, recomputation 67 -> 24, finish
+// (which formed the DG fluxes) 31 -> 11; every cell recomputed (mode 2), N = 5, 1e5 cells:
+// step 1.82 -> 1.55 ms.
+//
+// Both cells of a face between two troubled cells form its flux
 // from the same four subcell averages (P u^n of the same coefficients by the
 // same arithmetic), so they see the same bits.
 #pragma once
@@ -101,17 +106,21 @@ __device__ __forceinline__ void lim_subcell32(const LimParams& P, const float (&
   }
 }
 
-// per cell: FP32 extrema of the subcell averages of u^n and their bound
+// neighbour index with the boundary condition (-1: none, outflow boundary)
+__device__ __forceinline__ long long lim_neighbour(long long c, long long n, int bc) {
+  if (c >= 0 && c < n) return c;
+  if (bc == kBcOutflow) return -1;
+  return c < 0 ? c + n : c - n;
+}
+
+constexpr int kLimDetect = 128;               // threads of a detector block
+constexpr int kLimDetectCells = kLimDetect - 2;  // its cells (a halo cell at each end)
+
+// FP32 extrema of the subcell averages of u and their error bound
 template <int N>
-__global__ void __launch_bounds__(256) lim_minmax_kernel(const __grid_constant__ LimParams P) {
-  double dt;
-  int last;
-  if (!corrector_step_dt(P.sp, &dt, &last)) return;  // inactive step
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) P.sp.ctl->lim_n = 0;  // the detectors append to the list after this kernel
-  if (i >= P.ncells) return;
+__device__ __forceinline__ void lim_extrema32(const LimParams& P, const double* u, float* out) {
   float uf[N + 1][kM], bound[kM], lo[kM], hi[kM];
-  lim_image32<N>(P, P.u_old + i * ((N + 1) * kM), uf, bound);
+  lim_image32<N>(P, u, uf, bound);
 #pragma unroll
   for (int r = 0; r < kM; ++r) {
     lo[r] = INFINITY;
@@ -126,7 +135,6 @@ __global__ void __launch_bounds__(256) lim_minmax_kernel(const __grid_constant__
       hi[r] = fmaxf(hi[r], v[r]);
     }
   }
-  float* out = P.mmf + i * 9;
 #pragma unroll
   for (int r = 0; r < kM; ++r) {
     out[r] = lo[r];
@@ -135,37 +143,87 @@ __global__ void __launch_bounds__(256) lim_minmax_kernel(const __grid_constant__
   }
 }
 
-// neighbour index with the boundary condition (-1: none, outflow boundary)
-__device__ __forceinline__ long long lim_neighbour(long long c, long long n, int bc) {
-  if (c >= 0 && c < n) return c;
-  if (bc == kBcOutflow) return -1;
-  return c < 0 ? c + n : c - n;
+// NAD violated by one value (the FP64 detector)
+__device__ __forceinline__ bool lim_outside(double v, double lo, double hi, double delta) {
+  return v < lo - delta || v > hi + delta;
 }
 
+// the FP64 detectors of one cell by one thread
 template <int N>
-__global__ void __launch_bounds__(256) lim_detect_kernel(const __grid_constant__ LimParams P) {
+__device__ __noinline__ bool lim_detect64(const LimParams& P, long long i) {
+  double lo[kM], hi[kM];
+#pragma unroll
+  for (int r = 0; r < kM; ++r) {
+    lo[r] = INFINITY;
+    hi[r] = -INFINITY;
+  }
+  for (int d = -1; d <= 1; ++d) {
+    const long long c = lim_neighbour(i + d, P.ncells, P.bc);
+    if (c < 0) continue;
+    for (int j = 0; j < P.Ns; ++j) {
+      double v[kM];
+      lim_subcell<N>(P, P.u_old + c * ((N + 1) * kM), j, v);
+#pragma unroll
+      for (int r = 0; r < kM; ++r) {
+        lo[r] = fmin(lo[r], v[r]);
+        hi[r] = fmax(hi[r], v[r]);
+      }
+    }
+  }
+  double delta[kM];
+#pragma unroll
+  for (int r = 0; r < kM; ++r) delta[r] = fmax(P.delta0, P.eps * (hi[r] - lo[r]));
+  bool bad = false;
+  for (int j = 0; j < P.Ns; ++j) {
+    double v[kM];
+    lim_subcell<N>(P, P.u + i * ((N + 1) * kM), j, v);
+    if (!lim_admissible(v)) bad = true;
+#pragma unroll
+    for (int r = 0; r < kM; ++r)
+      if (lim_outside(v[r], lo[r], hi[r], delta[r])) bad = true;
+  }
+  return bad;
+}
+
+// A warp with more cells than this left to FP64 decides them itself, one lane each
+// (~1000 FP64 instructions for the warp); fewer are listed undecided and decided by
+// the blocks of lim_recompute_kernel (~140 warp instructions per cell, all SMs).  Step,
+// all in place / this / all listed: Sod tube, N = 5, 1e4 cells 169 / 130 / 130 us; NAD
+// with delta = 0 (nearly every cell), N = 3, 1e5 cells 1.49 / 1.49 / 1.57 ms.
+constexpr int kLimListed = 8;
+
+template <int N>
+__global__ void __launch_bounds__(kLimDetect)
+    lim_detect_kernel(const __grid_constant__ LimParams P) {
+  __shared__ float s_mm[kLimDetect][9];  // FP32 min, max of P u^n per variable, bound
   double dt;
   int last;
   if (!corrector_step_dt(P.sp, &dt, &last)) return;
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= P.ncells) return;
+  // thread t: the extrema of cell i; threads 1 .. kLimDetectCells also its screen
+  const int t = threadIdx.x;
+  const long long i = (long long)blockIdx.x * kLimDetectCells + t - 1;
+  const bool own = t >= 1 && t <= kLimDetectCells && i < P.ncells;
   if (P.mode == 2) {  // every cell recomputed on its subcells
-    P.troubled[i] = 1;
-    P.list[i] = i;
-    if (i == 0) {
-      P.sp.ctl->lim_n = (unsigned long long)P.ncells;
-      atomicAdd(&P.sp.ctl->troubled, (unsigned long long)P.ncells);
+    if (own) {
+      P.troubled[i] = 1;
+      P.list[i] = i;
+      if (i == 0) {
+        P.sp.ctl->lim_n = (unsigned long long)P.ncells;
+        atomicAdd(&P.sp.ctl->troubled, (unsigned long long)P.ncells);
+      }
     }
     return;
   }
+  const long long ci = i <= P.ncells ? lim_neighbour(i, P.ncells, P.bc) : -1;
+  if (ci >= 0) lim_extrema32<N>(P, P.u_old + ci * ((N + 1) * kM), s_mm[t]);
+  __syncthreads();
   // FP32 screen: the cell is certainly admissible when every FP32 subcell
   // average of u* lies inside the NAD interval and PAD holds with the error
-  // bounds to spare; otherwise the FP64 detectors below decide
-  const double* u = P.u + i * ((N + 1) * kM);
+  // bounds to spare; otherwise the FP64 detectors decide
   bool sure = true;
-  {
+  if (own) {
     float uf[N + 1][kM], bc[kM], lo[kM], hi[kM], bn[kM];
-    lim_image32<N>(P, u, uf, bc);
+    lim_image32<N>(P, P.u + i * ((N + 1) * kM), uf, bc);
 #pragma unroll
     for (int r = 0; r < kM; ++r) {
       lo[r] = INFINITY;
@@ -173,14 +231,13 @@ __global__ void __launch_bounds__(256) lim_detect_kernel(const __grid_constant__
       bn[r] = 0.f;
     }
     for (int d = -1; d <= 1; ++d) {
-      const long long c = lim_neighbour(i + d, P.ncells, P.bc);
-      if (c < 0) continue;
+      if (lim_neighbour(i + d, P.ncells, P.bc) < 0) continue;
+      const float* mm = s_mm[t + d];
 #pragma unroll
       for (int r = 0; r < kM; ++r) {
-        lo[r] = fminf(lo[r], P.mmf[c * 9 + r]);
-        hi[r] = fmaxf(hi[r], P.mmf[c * 9 + 3 + r]);
-        const float b = P.mmf[c * 9 + 6 + r];
-        bn[r] = b < 0.f ? INFINITY : fmaxf(bn[r], b);
+        lo[r] = fminf(lo[r], mm[r]);
+        hi[r] = fmaxf(hi[r], mm[3 + r]);
+        bn[r] = mm[6 + r] < 0.f ? INFINITY : fmaxf(bn[r], mm[6 + r]);
       }
     }
     float slack[kM], dlo[kM];
@@ -205,311 +262,309 @@ __global__ void __launch_bounds__(256) lim_detect_kernel(const __grid_constant__
       if (!(v[0] > 4.f * bc[0]) || !(v[2] - kin > 4.f * eb + 1e-6f * (fabsf(v[2]) + kin)))
         sure = false;
     }
+    if (sure) P.troubled[i] = 0;
   }
-  bool bad = false;
-  if (!sure) {
-    // FP64 detectors: extrema of the cell and its neighbours from u^n, then PAD
-    // and NAD on the subcell averages of u*
-    double lo[kM], hi[kM];
-#pragma unroll
-    for (int r = 0; r < kM; ++r) {
-      lo[r] = INFINITY;
-      hi[r] = -INFINITY;
-    }
-    for (int d = -1; d <= 1; ++d) {
-      const long long c = lim_neighbour(i + d, P.ncells, P.bc);
-      if (c < 0) continue;
-      for (int j = 0; j < P.Ns; ++j) {
-        double v[kM];
-        lim_subcell<N>(P, P.u_old + c * ((N + 1) * kM), j, v);
-#pragma unroll
-        for (int r = 0; r < kM; ++r) {
-          lo[r] = fmin(lo[r], v[r]);
-          hi[r] = fmax(hi[r], v[r]);
-        }
-      }
-    }
-    double delta[kM];
-#pragma unroll
-    for (int r = 0; r < kM; ++r) delta[r] = fmax(P.delta0, P.eps * (hi[r] - lo[r]));
-    for (int j = 0; j < P.Ns; ++j) {
-      double v[kM];
-      lim_subcell<N>(P, u, j, v);
-      if (!lim_admissible(v)) bad = true;
-#pragma unroll
-      for (int r = 0; r < kM; ++r)
-        if (v[r] < lo[r] - delta[r] || v[r] > hi[r] + delta[r]) bad = true;
-    }
-  }
-  P.troubled[i] = bad ? 1 : 0;
-  if (bad) {
+  const bool here = __popc(__ballot_sync(0xffffffffu, !sure)) > kLimListed;  // uniform
+  if (sure) return;
+  if (here) {
+    const bool bad = lim_detect64<N>(P, i);
+    P.troubled[i] = bad ? 1 : 0;
+    if (!bad) return;
     atomicAdd(&P.sp.ctl->troubled, 1ull);
-    P.list[atomicAdd(&P.sp.ctl->lim_n, 1ull)] = i;
   }
+  P.list[atomicAdd(&P.sp.ctl->lim_n, 1ull)] = here ? i : ~i;  // ~i: not decided yet
 }
 
-// DG face flux (time-integrated, rescaled) from the predictor traces, as the
-// interface kernel forms it: (dt/dx)/2 sum_l0 w_l0 (2 G)(qR_left, qL_right).
-template <int N>
-__device__ __forceinline__ void lim_dg_face(const LimParams& P, long long f, double hlam,
-                                            double* G) {
-  constexpr int n = N + 1, stride = 9 * n;
-  const long long cl = lim_neighbour(f - 1, P.ncells, P.bc), cr = lim_neighbour(f, P.ncells, P.bc);
-  // outflow boundary: the ghost side holds the boundary cell's mean of u^n
-  double ghost[kM];
-  if (cl < 0 || cr < 0) {
-    const long long cb = cl < 0 ? cr : cl;
-#pragma unroll
-    for (int r = 0; r < kM; ++r) {
-      double m = 0.0;
-#pragma unroll
-      for (int k = 0; k < n; ++k) m = fma(P.ops.w[k], P.u_old[(cb * n + k) * kM + r], m);
-      ghost[r] = m;
-    }
-  }
-  double s[kM] = {0.0, 0.0, 0.0};
-#pragma unroll
-  for (int l0 = 0; l0 < n; ++l0) {
-    const double* ta = cl >= 0 ? P.trace + cl * stride + l0 * kM : ghost;
-    const double* tb = cr >= 0 ? P.trace + cr * stride + n * kM + l0 * kM : ghost;
-    double a[kM], b[kM], G2[kM];
-#pragma unroll
-    for (int r = 0; r < kM; ++r) {
-      a[r] = ta[r];
-      b[r] = tb[r];
-    }
-    rusanov2(a, b, G2, P.gamma, P.gm1);
-#pragma unroll
-    for (int r = 0; r < kM; ++r) s[r] = fma(P.ops.w[l0], G2[r], s[r]);
-  }
-#pragma unroll
-  for (int r = 0; r < kM; ++r) G[r] = hlam * s[r];
-}
-
-// Degree-1 WENO on a subcell with averages v0 and neighbours vm, vp: slopes of
-// the stencils {j-1, j} and {j, j+1}, smoothness sigma_S = slope_S^2, weights
-// (sigma_S + 1e-14)^-8 normalised (written as 1 / (1 + (s_l / s_r)^8)), nodal
-// values at the two Gauss nodes.
-__device__ __forceinline__ void lim_weno2(const Sub1Ops& s1, const double* vm, const double* v0,
-                                          const double* vp, double (*w)[kM]) {
-#pragma unroll
-  for (int r = 0; r < kM; ++r) {
-    const double sl = v0[r] - vm[r], sr = vp[r] - v0[r];
-    double t = fma(sl, sl, 1.0e-14) / fma(sr, sr, 1.0e-14);
-    t *= t;
-    t *= t;
-    t *= t;
-    const double om = 1.0 / (1.0 + t);  // weight of the left stencil
-    const double slope = fma(om, sl - sr, sr);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) w[k][r] = fma(slope, s1.xi[k] - 0.5, v0[r]);
-  }
+// Degree-1 WENO slope of one variable on a subcell with average v0 and neighbours vm,
+// vp: slopes of the stencils {j-1, j} and {j, j+1}, smoothness sigma_S = slope_S^2,
+// weights (sigma_S + 1e-14)^-8 normalised (written as 1 / (1 + (s_l / s_r)^8)).
+__device__ __forceinline__ double lim_slope(double vm, double v0, double vp) {
+  const double sl = v0 - vm, sr = vp - v0;
+  double t = fma(sl, sl, 1.0e-14) * rcp64(fma(sr, sr, 1.0e-14));
+  t *= t;
+  t *= t;
+  t *= t;
+  const double om = rcp64(1.0 + t);  // weight of the left stencil
+  return fma(om, sl - sr, sr);
 }
 
 // LST-DG predictor of degree 1 on one subcell (eq. lst_dg_predictor_picard with
-// the degree-1 operators; lam_s = dt / subcell width) and its traces at both ends
-// at the two tau nodes.  Convergence as the DG predictor: max |q' - q| <=
-// tol max(1, max |q'|), capped by max_iter; fixed_iter > 0 runs exactly that many.
+// the degree-1 operators; lam_s = dt / subcell width) by four lanes, lane p = 2 p0 + p1
+// holding the node (tau p0, xi p1) and w its initial value; then the traces at the tau
+// node p0: at xi = 1 (p1 = 0) or xi = 0 (p1 = 1).  Convergence as the DG predictor:
+// max |q' - q| <= tol max(1, max |q'|), capped by max_iter; fixed_iter > 0 runs exactly
+// that many.  Called by whole warps; `idle` lanes take part in the exchanges only.
 __device__ __forceinline__ bool lim_predict1(const LimParams& P, double lam_s,
-                                             const double (*w)[kM], double (*qR)[kM],
-                                             double (*qL)[kM]) {
+                                             const double (&w)[kM], bool idle, double* trace) {
   const Sub1Ops& s1 = P.s1;
-  double q[2][2][kM];
-#pragma unroll
-  for (int p0 = 0; p0 < 2; ++p0)
-#pragma unroll
-    for (int p1 = 0; p1 < 2; ++p1)
-#pragma unroll
-      for (int r = 0; r < kM; ++r) q[p0][p1][r] = w[p1][r];
-  const int cap = P.fixed_iter > 0 ? P.fixed_iter : P.max_iter;
-  bool converged = P.fixed_iter > 0;
+  const int p1 = threadIdx.x & 1, p0 = (threadIdx.x >> 1) & 1;
+  constexpr unsigned all = 0xffffffffu;
+  // own and exchanged operands: (dt / dx) k~ by xi, then -kappa~ by tau
+  const double kto = lam_s * s1.kt[p1][p1], ktx = lam_s * s1.kt[p1][p1 ^ 1];
+  const double kao = -s1.kap[p0][p0], kax = -s1.kap[p0][p0 ^ 1];
+  auto magnitude = [](double x) {  // the bit pattern of |x|; a NaN does not count (as fmax)
+    const unsigned long long b = dbits(x) & 0x7fffffffffffffffull;
+    return b > 0x7ff0000000000000ull ? 0ull : b;
+  };
+  double q[kM] = {w[0], w[1], w[2]};
+  const bool fixed = P.fixed_iter > 0;
+  const int cap = fixed ? P.fixed_iter : P.max_iter;
+  bool done = idle, converged = fixed || idle;
   for (int it = 0; it < cap; ++it) {
-    double f[2][2][kM];
-#pragma unroll
-    for (int p0 = 0; p0 < 2; ++p0)
-#pragma unroll
-      for (int p1 = 0; p1 < 2; ++p1) {
-        euler_flux<double>(q[p0][p1], f[p0][p1], P.gm1);
-#pragma unroll
-        for (int r = 0; r < kM; ++r) f[p0][p1][r] *= lam_s;
-      }
-    double sx[2][2][kM];
-#pragma unroll
-    for (int p0 = 0; p0 < 2; ++p0)
-#pragma unroll
-      for (int p1 = 0; p1 < 2; ++p1)
-#pragma unroll
-        for (int r = 0; r < kM; ++r)
-          sx[p0][p1][r] = fma(s1.kt[p1][0], f[p0][0][r], s1.kt[p1][1] * f[p0][1][r]);
-    double delta = 0.0, qmax = 0.0;
-#pragma unroll
-    for (int p0 = 0; p0 < 2; ++p0)
-#pragma unroll
-      for (int p1 = 0; p1 < 2; ++p1)
-#pragma unroll
-        for (int r = 0; r < kM; ++r) {
-          const double qn =
-              w[p1][r] - fma(s1.kap[p0][0], sx[0][p1][r], s1.kap[p0][1] * sx[1][p1][r]);
-          delta = fmax(delta, fabs(qn - q[p0][p1][r]));
-          qmax = fmax(qmax, fabs(qn));
-          q[p0][p1][r] = qn;
-        }
-    if (P.fixed_iter <= 0 && delta <= P.tol * fmax(qmax, 1.0)) {
-      converged = true;
-      break;
-    }
-  }
-#pragma unroll
-  for (int l0 = 0; l0 < 2; ++l0)
+    double f[kM], qn[kM];
+    euler_flux<double>(q, f, P.gm1);
+    unsigned long long delta = 0ull, qmax = 0ull;
 #pragma unroll
     for (int r = 0; r < kM; ++r) {
-      qR[l0][r] = fma(s1.psi1[0], q[l0][0][r], s1.psi1[1] * q[l0][1][r]);
-      qL[l0][r] = fma(s1.psi0[0], q[l0][0][r], s1.psi0[1] * q[l0][1][r]);
+      const double sx = fma(kto, f[r], ktx * __shfl_xor_sync(all, f[r], 1));
+      qn[r] = fma(kao, sx, fma(kax, __shfl_xor_sync(all, sx, 2), w[r]));
+      delta = umax64(delta, magnitude(qn[r] - q[r]));
+      qmax = umax64(qmax, magnitude(qn[r]));
     }
+#pragma unroll
+    for (int m = 1; m <= 2; m <<= 1) {
+      delta = umax64(delta, __shfl_xor_sync(all, delta, m));
+      qmax = umax64(qmax, __shfl_xor_sync(all, qmax, m));
+    }
+    if (!done) {
+#pragma unroll
+      for (int r = 0; r < kM; ++r) q[r] = qn[r];
+      if (!fixed && bitsd(delta) <= P.tol * bitsd(umax64(qmax, dbits(1.0)))) done = converged = true;
+    }
+    if (__all_sync(all, done)) break;
+  }
+  const double* psi = p1 ? s1.psi0 : s1.psi1;
+  const double pso = psi[p1], psx = psi[p1 ^ 1];
+#pragma unroll
+  for (int r = 0; r < kM; ++r) trace[r] = fma(pso, q[r], psx * __shfl_xor_sync(all, q[r], 1));
   return converged;
 }
 
-constexpr int kLimWarps = 4;  // warps (listed cells in flight) per block
+template <int N>
+struct LimCfg {
+  static constexpr int n = N + 1, Ns = 2 * N + 1;
+  // four lanes per subcell, the neighbours' boundary subcells included
+  static constexpr int THREADS = (4 * (Ns + 2) + 31) / 32 * 32;
+  static constexpr int FLUXES = 2 * (Ns + 1) + 2 * n;  // (subcell face, tau) | (side, tau)
+};
 
 template <int N>
-struct LimWarpSmem {
+struct LimSmem {
   static constexpr int n = N + 1, Ns = 2 * N + 1;
+  double P[Ns][n], R[n][Ns];
+  double v[3][Ns][kM];       // P u^n of the left neighbour, the cell, the right neighbour
+  double lo[kM], hi[kM];
   double ve[Ns + 4][kM];     // subcell averages of u^n, subcells -2 .. Ns+1
-  double qR[Ns + 2][2][kM];  // traces of subcells -1 .. Ns at the two tau nodes
-  double qL[Ns + 2][2][kM];
+  double tr[Ns + 2][2][2][kM];  // traces of subcells -1 .. Ns: [tau][at xi = 1, 0]
+  double G[LimCfg<N>::FLUXES][kM];
   double F[Ns + 1][kM];      // subcell face fluxes (dt/dx scaling)
-  double vnew[Ns][kM];
+  double vnew[Ns][kM];       // (the detectors: P u*)
   double ur[n][kM];
 };
 
-// Two listed cells per warp, one per half-warp group of kLimGroup lanes: the
-// degree-1 subcell predictors (Ns + 2 per cell, 13 at N = 5) would otherwise
-// leave most of a warp idle, and the FP64 pipe issues whole warps.  Phases wider
-// than a group (the predictors at N = 7, the (k, r) reconstruction lanes) loop
-// with the group's stride; the admissibility vote is per group.
-constexpr int kLimGroup = 16;
-
 template <int N>
-__global__ void __launch_bounds__(32 * kLimWarps)
+__global__ void __launch_bounds__(LimCfg<N>::THREADS)
     lim_recompute_kernel(const __grid_constant__ LimParams P) {
-  constexpr int n = N + 1, Ns = 2 * N + 1, G = kLimGroup;
-  __shared__ LimWarpSmem<N> smem[2 * kLimWarps];
+  constexpr int n = N + 1, Ns = 2 * N + 1, T = LimCfg<N>::THREADS, stride = 9 * n;
+  __shared__ LimSmem<N> sh;
   double dt;
   int last;
   if (!corrector_step_dt(P.sp, &dt, &last)) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int grp = lane / G, l = lane - grp * G;
-  const unsigned gmask = grp ? 0xffff0000u : 0x0000ffffu;
-  LimWarpSmem<N>& w = smem[2 * warp + grp];
+  const int tid = threadIdx.x;
   const long long count = (long long)P.sp.ctl->lim_n;
+  if (blockIdx.x >= count) return;
+  for (int t = tid; t < Ns * n; t += T) {
+    (&sh.P[0][0])[t] = P.ops.P[t / n][t % n];
+    (&sh.R[0][0])[t] = P.R[t / Ns][t % Ns];
+  }
   const double hlam = 0.5 * dt * P.sp.inv_dx;
   const double lam_s = dt * P.sp.inv_dx * (double)Ns;  // dt / subcell width
-  // the loop runs over cell pairs, uniform over the warp (a group without a
-  // cell in the last pair idles through the warp's synchronisations)
-  for (long long pe = (long long)blockIdx.x * kLimWarps + warp; 2 * pe < count;
-       pe += (long long)gridDim.x * kLimWarps) {
-    const long long e = 2 * pe + grp;
-    const bool has = e < count;
-    const long long i = has ? P.list[e] : 0;
-    const long long il = lim_neighbour(i - 1, P.ncells, P.bc), ir = lim_neighbour(i + 1, P.ncells, P.bc);
-    // subcell averages of u^n: the cell's own, and the neighbours' two subcells
-    // next to each face (l = 0, 1: left neighbour's Ns-2, Ns-1; l = 2, 3: right
-    // neighbour's 0, 1), by the same arithmetic the neighbour uses for its own,
+  for (long long e = blockIdx.x; e < count; e += gridDim.x) {
+    const long long entry = P.list[e], i = entry < 0 ? ~entry : entry;
+    const long long nb[2] = {lim_neighbour(i - 1, P.ncells, P.bc),
+                             lim_neighbour(i + 1, P.ncells, P.bc)};
+    __syncthreads();  // the tables; the last cell's shared memory
+    // subcell averages of u^n of the three cells: every cell's by the same arithmetic,
     // so both sides of a face between troubled cells see the same bits
-    if (has) {
-      for (int j = l; j < Ns; j += G) lim_subcell<N>(P, P.u_old + i * (n * kM), j, w.ve[j + 2]);
-      if (l < 4) {
-        const long long nb = l < 2 ? il : ir;
-        if (nb >= 0)
-          lim_subcell<N>(P, P.u_old + nb * (n * kM), l < 2 ? Ns - 2 + l : l - 2,
-                         w.ve[l < 2 ? l : Ns + l]);
-      }
-    }
-    __syncwarp();
-    if (has && l < 4) {  // outflow boundary: the boundary subcell itself
-      const long long nb = l < 2 ? il : ir;
-      if (nb < 0) {
+    for (int t = tid; t < 3 * Ns * kM; t += T) {
+      const int d = t / (Ns * kM), j = t / kM - d * Ns, r = t % kM;
+      const long long c = d == 1 ? i : nb[d >> 1];
+      double acc = 0.0;
+      if (c >= 0) {
 #pragma unroll
-        for (int r = 0; r < kM; ++r) w.ve[l < 2 ? l : Ns + l][r] = w.ve[l < 2 ? 2 : Ns + 1][r];
+        for (int k = 0; k < n; ++k) acc = fma(sh.P[j][k], P.u_old[(c * n + k) * kM + r], acc);
       }
+      sh.v[d][j][r] = acc;
     }
-    __syncwarp();
-    // item j: subcell j - 1 (ve index j + 1): degree-1 WENO and predictor
-    if (has) {
-      for (int j = l; j < Ns + 2; j += G) {
-        double wn[2][kM];
-        lim_weno2(P.s1, w.ve[j], w.ve[j + 1], w.ve[j + 2], wn);
-        if (!lim_predict1(P, lam_s, wn, w.qR[j], w.qL[j]))
-          atomicOr(&P.sp.ctl->status, kStNotConverged);
-      }
-    }
-    __syncwarp();
-    // item f: face between subcells f - 1 and f
-    if (has) {
-      for (int f = l; f < Ns + 1; f += G) {
-        double s[kM] = {0.0, 0.0, 0.0};
-#pragma unroll
-        for (int l0 = 0; l0 < 2; ++l0) {
-          double G2[kM];
-          rusanov2(w.qR[f][l0], w.qL[f + 1][l0], G2, P.gamma, P.gm1);
-#pragma unroll
-          for (int r = 0; r < kM; ++r) s[r] = fma(P.s1.w[l0], G2[r], s[r]);
+    __syncthreads();
+    if (entry < 0) {
+      // FP64 detectors: extrema of the cell and its neighbours from u^n, then PAD
+      // and NAD on the subcell averages of u*
+      if (tid < 32) {
+        const int r = tid >> 3, s = tid & 7;  // eight lanes per variable
+        double lo = INFINITY, hi = -INFINITY;
+        if (r < kM) {
+          for (int t = s; t < 3 * Ns; t += 8) {
+            const int d = t / Ns;
+            if (d != 1 && nb[d >> 1] < 0) continue;
+            const double v = sh.v[d][t - d * Ns][r];
+            lo = fmin(lo, v);
+            hi = fmax(hi, v);
+          }
         }
 #pragma unroll
-        for (int r = 0; r < kM; ++r) {
-          w.F[f][r] = hlam * s[r];
-          if (f == 0) P.gface[i * 6 + r] = hlam * s[r];
-          if (f == Ns) P.gface[i * 6 + 3 + r] = hlam * s[r];
+        for (int m = 1; m < 8; m <<= 1) {
+          lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, m));
+          hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, m));
+        }
+        if (r < kM && s == 0) {
+          const double delta = fmax(P.delta0, P.eps * (hi - lo));
+          sh.lo[r] = lo - delta;
+          sh.hi[r] = hi + delta;
         }
       }
-    }
-    __syncwarp();
-    if (has) {
-      for (int j = l; j < Ns; j += G) {
-#pragma unroll
-        for (int r = 0; r < kM; ++r)
-          w.vnew[j][r] = w.ve[j + 2][r] - (double)Ns * (w.F[j + 1][r] - w.F[j][r]);
-      }
-    }
-    __syncwarp();
-    // reconstruction u = R v (item = (k, r))
-    if (has) {
-      for (int t = l; t < n * kM; t += G) {
-        const int k = t / kM, r = t - k * kM;
+      for (int t = tid; t < Ns * kM; t += T) {
+        const int j = t / kM, r = t % kM;
         double acc = 0.0;
-        for (int j = 0; j < Ns; ++j) acc = fma(P.R[k][j], w.vnew[j][r], acc);
-        w.ur[k][r] = acc;
+#pragma unroll
+        for (int k = 0; k < n; ++k) acc = fma(sh.P[j][k], P.u[(i * n + k) * kM + r], acc);
+        sh.vnew[j][r] = acc;
+      }
+      __syncthreads();
+      bool bad = false;
+      for (int t = tid; t < Ns * (kM + 1); t += T) {  // NAD per value, then PAD per subcell
+        if (t < Ns * kM) {
+          const double v = sh.vnew[t / kM][t % kM];
+          bad = bad || v < sh.lo[t % kM] || v > sh.hi[t % kM];
+        } else {
+          bad = bad || !lim_admissible(sh.vnew[t - Ns * kM]);
+        }
+      }
+      const bool any = __syncthreads_or(bad);
+      if (tid == 0) {
+        P.troubled[i] = any ? 1 : 0;
+        if (any) atomicAdd(&P.sp.ctl->troubled, 1ull);
+      }
+      if (!any) continue;  // uniform
+    }
+    // the cell's subcells and the neighbours' two next to each face (outflow
+    // boundary: the boundary subcell itself)
+    for (int t = tid; t < (Ns + 4) * kM; t += T) {
+      const int j = t / kM - 2, r = t % kM;
+      const int side = j < 0 ? 0 : 2;
+      double v;
+      if (j >= 0 && j < Ns)
+        v = sh.v[1][j][r];
+      else if (nb[side >> 1] >= 0)
+        v = sh.v[side][j < 0 ? Ns + j : j - Ns][r];
+      else
+        v = sh.v[1][j < 0 ? 0 : Ns - 1][r];
+      sh.ve[j + 2][r] = v;
+    }
+    __syncthreads();
+    {
+      // subcell s - 1 by lanes 4 s .. 4 s + 3: the slope's variables spread over the
+      // lanes, then the predictor
+      const int s = tid >> 2, sc = s < Ns + 2 ? s : Ns + 1, l = tid & 3;
+      const int rs = l < kM ? l : 0;
+      const double slope = lim_slope(sh.ve[sc][rs], sh.ve[sc + 1][rs], sh.ve[sc + 2][rs]);
+      double w[kM], tr[kM];
+#pragma unroll
+      for (int r = 0; r < kM; ++r)
+        w[r] = fma(__shfl_sync(0xffffffffu, slope, (tid & 28) | r), P.s1.xi[l & 1] - 0.5,
+                   sh.ve[sc + 1][r]);
+      const bool ok = lim_predict1(P, lam_s, w, s > Ns + 1, tr);
+      if (s <= Ns + 1) {
+        if (!ok) atomicOr(&P.sp.ctl->status, kStNotConverged);
+#pragma unroll
+        for (int r = 0; r < kM; ++r) sh.tr[s][l >> 1][l & 1][r] = tr[r];
       }
     }
-    __syncwarp();
-    bool ok = true;
-    if (has) {
-      for (int j = l; j < Ns; j += G) {
-        double v[kM];
+    __syncthreads();
+    // Rusanov fluxes: item (f, l0) of the subcell faces (f between subcells f - 1 and
+    // f), then (side, l0) of the cell's own faces from the DG predictor's traces
+    // (mode 2 has no cell that would use the latter)
+    const int fluxes = P.mode == 2 ? 2 * (Ns + 1) : LimCfg<N>::FLUXES;
+    for (int t = tid; t < fluxes; t += T) {
+      double a[kM], b[kM], G2[kM];
+      if (t < 2 * (Ns + 1)) {
 #pragma unroll
         for (int r = 0; r < kM; ++r) {
-          double acc = 0.0;
+          a[r] = sh.tr[t >> 1][t & 1][0][r];
+          b[r] = sh.tr[(t >> 1) + 1][t & 1][1][r];
+        }
+      } else {
+        const int side = (t - 2 * (Ns + 1)) / n, l0 = t - 2 * (Ns + 1) - side * n;
+        const long long cl = side ? i : nb[0], cr = side ? nb[1] : i;
+        if (cl < 0 || cr < 0) {
+          // outflow boundary: the ghost side holds the boundary cell's mean of u^n
 #pragma unroll
-          for (int k = 0; k < n; ++k) acc = fma(P.ops.P[j][k], w.ur[k][r], acc);
-          v[r] = acc;
+          for (int r = 0; r < kM; ++r) {
+            double m = 0.0;
+#pragma unroll
+            for (int k = 0; k < n; ++k) m = fma(P.ops.w[k], P.u_old[(i * n + k) * kM + r], m);
+            a[r] = b[r] = m;
+          }
         }
-        ok = ok && lim_admissible(v);
+#pragma unroll
+        for (int r = 0; r < kM; ++r) {
+          if (cl >= 0) a[r] = P.trace[cl * stride + l0 * kM + r];
+          if (cr >= 0) b[r] = P.trace[cr * stride + (n + l0) * kM + r];
+        }
+      }
+      rusanov2(a, b, G2, P.gamma, P.gm1);
+#pragma unroll
+      for (int r = 0; r < kM; ++r) sh.G[t][r] = G2[r];
+    }
+    __syncthreads();
+    for (int t = tid; t < (Ns + 1) * kM; t += T) {
+      const int f = t / kM, r = t - f * kM;
+      const double F =
+          hlam * fma(P.s1.w[1], sh.G[2 * f + 1][r], P.s1.w[0] * sh.G[2 * f][r]);
+      sh.F[f][r] = F;
+      if (P.mode != 2 && (f == 0 || f == Ns)) {
+        const int side = f ? 1 : 0;
+        double g = 0.0;
+#pragma unroll
+        for (int l0 = 0; l0 < n; ++l0)
+          g = fma(P.ops.w[l0], sh.G[2 * (Ns + 1) + side * n + l0][r], g);
+        P.gface[i * 6 + side * kM + r] = F - hlam * g;
       }
     }
-    ok = (__ballot_sync(0xffffffffu, !ok) & gmask) == 0u;  // this group's vote
-    if (has) {
-      for (int t = l; t < n * kM; t += G) {
-        const int k = t / kM, r = t - k * kM;
-        double val = w.ur[k][r];
-        if (!ok) {  // the mean of the subcell values
-          double mean = 0.0;
-          for (int j = 0; j < Ns; ++j) mean += w.vnew[j][r];
-          val = mean / (double)Ns;
-        }
-        P.u[(i * n + k) * kM + r] = val;
-      }
+    __syncthreads();
+    for (int t = tid; t < Ns * kM; t += T) {
+      const int j = t / kM, r = t - j * kM;
+      sh.vnew[j][r] = sh.ve[j + 2][r] - (double)Ns * (sh.F[j + 1][r] - sh.F[j][r]);
     }
-    __syncwarp();  // shared memory is free for the next pair
+    __syncthreads();
+    // reconstruction u = R v (item = (k, r))
+    for (int t = tid; t < n * kM; t += T) {
+      const int k = t / kM, r = t - k * kM;
+      double acc = 0.0;
+#pragma unroll
+      for (int j = 0; j < Ns; ++j) acc = fma(sh.R[k][j], sh.vnew[j][r], acc);
+      sh.ur[k][r] = acc;
+    }
+    __syncthreads();
+    for (int t = tid; t < Ns * kM; t += T) {
+      const int j = t / kM, r = t - j * kM;
+      double acc = 0.0;
+#pragma unroll
+      for (int k = 0; k < n; ++k) acc = fma(sh.P[j][k], sh.ur[k][r], acc);
+      sh.v[0][j][r] = acc;
+    }
+    __syncthreads();
+    const bool ok = __syncthreads_and(tid >= Ns || lim_admissible(sh.v[0][tid < Ns ? tid : 0]));
+    for (int t = tid; t < n * kM; t += T) {
+      const int k = t / kM, r = t - k * kM;
+      double val = sh.ur[k][r];
+      if (!ok) {  // the mean of the subcell values
+        double mean = 0.0;
+        for (int j = 0; j < Ns; ++j) mean += sh.vnew[j][r];
+        val = mean / (double)Ns;
+      }
+      P.u[(i * n + k) * kM + r] = val;
+    }
   }
 }
 
@@ -531,6 +586,7 @@ __global__ void __launch_bounds__(128) lim_finish_kernel(const __grid_constant__
   int last;
   if (!corrector_step_dt(P.sp, &dt, &last)) return;  // uniform over the grid
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) P.sp.ctl->lim_n = 0;  // for the next step (the control block starts zeroed)
   const bool valid = i < P.ncells;
   double u[n][kM];
   if (valid) {
@@ -543,18 +599,14 @@ __global__ void __launch_bounds__(128) lim_finish_kernel(const __grid_constant__
       const long long il = lim_neighbour(i - 1, P.ncells, P.bc), ir = lim_neighbour(i + 1, P.ncells, P.bc);
       const bool tl = il >= 0 && P.troubled[il], tr = ir >= 0 && P.troubled[ir];
       if (tl || tr) {
-        const double hlam = 0.5 * dt * P.sp.inv_dx;
-        double GL[kM], GR[kM];
-        if (tl) lim_dg_face<N>(P, i, hlam, GL);
-        if (tr) lim_dg_face<N>(P, i + 1, hlam, GR);
 #pragma unroll
         for (int k = 0; k < n; ++k)
 #pragma unroll
           for (int r = 0; r < kM; ++r) {
             double d = 0.0;
-            if (tr) d -= P.ops.psi1[k] * (P.gface[ir * 6 + r] - GR[r]);
-            if (tl) d += P.ops.psi0[k] * (P.gface[il * 6 + 3 + r] - GL[r]);
-            u[k][r] += d / P.ops.w[k];
+            if (tr) d -= P.ops.psi1[k] * P.gface[ir * 6 + r];
+            if (tl) d += P.ops.psi0[k] * P.gface[il * 6 + 3 + r];
+            u[k][r] = fma(d, P.ops.rw[k], u[k][r]);
             up[k * kM + r] = u[k][r];
           }
       }
