@@ -373,7 +373,7 @@ ader_status ader_get_troubled(ader_ctx* ctx, int32_t* flags_dev, int64_t count);
 typedef struct {
   int predict_cells_per_block;  /* predictor tile: 16, 32 or 64 cells x (N+1) threads; the FP64
                                    form's fixed-point kernel: 2, 4 or 8 warps of 32 / (N+1) cells */
-  int face_cells_per_block;     /* interface/update tile: 32 or 64 cells per 256 threads */
+  int face_cells_per_block;     /* interface/update tile: the cells between 32 or 64 faces */
   int graph_steps;              /* time steps per CUDA-graph replay in ader_solve (even, 2..64) */
   double predict_ms;            /* measured per launch for the chosen shape (autotune only) */
   double face_ms;

@@ -297,7 +297,7 @@ cudaError_t launch_predict_nc(const PredictParams& p, cudaStream_t s) {
 
 cudaError_t launch_face_nc(const FaceParams& p, cudaStream_t s) {
   using C = FaceCfg<D, 32>;
-  const long long blocks = (p.ncells + C::C - 1) / C::C;
+  const long long blocks = (p.ncells + C::CELLS - 1) / C::CELLS;
   if (blocks <= 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   face_nc_kernel<D, 32><<<(unsigned)blocks, C::THREADS, 0, s>>>(p);
   return cudaGetLastError();
@@ -305,7 +305,7 @@ cudaError_t launch_face_nc(const FaceParams& p, cudaStream_t s) {
 
 cudaError_t launch_face_src(const FaceParams& p, cudaStream_t s) {
   using C = FaceCfg<D, 32>;
-  const long long blocks = (p.ncells + C::C - 1) / C::C;
+  const long long blocks = (p.ncells + C::CELLS - 1) / C::CELLS;
   if (blocks <= 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   face_src_kernel<D, 32><<<(unsigned)blocks, C::THREADS, 0, s>>>(p);
   return cudaGetLastError();
@@ -314,7 +314,7 @@ cudaError_t launch_face_src(const FaceParams& p, cudaStream_t s) {
 template <int CF>
 cudaError_t launch_face_cf(const FaceParams& p, cudaStream_t s) {
   using C = FaceCfg<D, CF>;
-  const long long blocks = (p.ncells + C::C - 1) / C::C;
+  const long long blocks = (p.ncells + C::CELLS - 1) / C::CELLS;
   if (blocks <= 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   face_update_kernel<D, CF><<<(unsigned)blocks, C::THREADS, 0, s>>>(p);
   return cudaGetLastError();

@@ -137,6 +137,17 @@ __device__ __forceinline__ void corrector_finish(const StepParams& sp, double dt
   }
 }
 
+// asynchronous copy of 8 bytes, global to shared (both 8-byte aligned)
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // ---- 1D Euler (rho, m = rho u, E) ----
 
 // 1/x in FP64 within one unit in the last place of 1.0 / x: a float seed

@@ -894,19 +894,24 @@ __global__ void __launch_bounds__(PredCfg<N, CPB>::THREADS)
   }
 }
 
-// Interface/update tile: C cells per 256-thread block (tuning choice: 32 or 64).
+// Interface/update tile: the cells between C faces (tuning choice: 32 or 64).
 template <int N, int C_ = 64>
 struct FaceCfg {
   static constexpr int n = N + 1;
-  static constexpr int C = C_;
-  static constexpr int THREADS = 256;
+  static constexpr int C = C_;          // faces of a tile; its cells lie between them
+  static constexpr int CELLS = C - 1;
+  // whole passes over the C n (face, tau) items: one, or two from n = 5 with 64 faces
+  static constexpr int THREADS = C == 64 && n <= 4 ? 64 * n : 32 * n;
+  // 64 registers: fewer spill the fixed-point flux (71-74), more leave too few warps
+  // for the short phases between barriers
+  static constexpr int MIN_BLOCKS = 1024 / THREADS;
 };
 
 template <int N, int C = 64>
 struct FaceShared {
-  double G[(C + 1) * (N + 1) * kM];
-  double Gs[(C + 1) * kM];
-  double u[C * (N + 1) * kM];
+  double G[C * (N + 1) * kM];
+  double Gs[C * kM];
+  double u[C * (N + 1) * kM];  // u + volume term (DG) or u^n (FV), then the new state
   double P[(2 * N + 1) * (N + 1)];
   double w[N + 1], psi0w[N + 1], psi1w[N + 1];  // w, psi_k / w_k, psi~_k / w_k
   float lt[C * (2 * N + 1)];        // FP32 upper bound of each subcell's speed (CFL)
@@ -1148,30 +1153,66 @@ __device__ __forceinline__ void rusanov2_screened(const double* a, const double*
   G2[2] = fma(-s, d2, F2);
 }
 
-// One tile (C cells) of the interface flux + update (+ lambda_max) of one solve.
+// What a tile needs from memory, asked for before anything waits: each cell's u + volume
+// term (DG) or average (FV) by asynchronous copies into sh.u, the traces of the thread's
+// first (face, tau) item into a, b.
+template <int N, int C>
+__device__ __forceinline__ int face_valid(const FaceIO& io, long long tile) {
+  constexpr int CELLS = FaceCfg<N, C>::CELLS;
+  const long long c0 = tile * CELLS;
+  return (int)((io.ncells - c0) < CELLS ? (io.ncells - c0) : CELLS);
+}
+template <int N>
+__device__ __forceinline__ void face_traces(const FaceParams& P, const FaceIO& io, long long c0,
+                                            int item, double (&a)[kM], double (&b)[kM]) {
+  constexpr int n = N + 1;
+  const int stride = (P.dg ? 9 : 6) * n;
+  const int f = item / n, l0 = item - f * n;
+  const long long cl = wrap_cell(c0 + f - 1, io.ncells), cr = wrap_cell(c0 + f, io.ncells);
+  const double* ta = io.trace + cl * stride + l0 * kM;           // qR of the left cell
+  const double* tb = io.trace + cr * stride + n * kM + l0 * kM;  // qL of the right cell
+#pragma unroll
+  for (int r = 0; r < kM; ++r) {
+    a[r] = ta[r];
+    b[r] = tb[r];
+  }
+}
+template <int N, int C>
+__device__ __forceinline__ void face_prefetch(const FaceParams& P, const FaceIO& io, long long tile,
+                                              FaceShared<N, C>& sh, double (&a)[kM],
+                                              double (&b)[kM]) {
+  constexpr int n = N + 1, THREADS = FaceCfg<N, C>::THREADS;
+  const long long c0 = tile * FaceCfg<N, C>::CELLS;
+  const int nvalid = face_valid<N, C>(io, tile), tid = threadIdx.x;
+  if (P.dg) {
+    const double* up = io.trace + c0 * (9 * n) + 2 * n * kM;
+    for (int i = tid; i < nvalid * n * kM; i += THREADS) {
+      const int lc = i / (n * kM);
+      cp_async8(&sh.u[i], up + (long long)lc * (9 * n) + (i - lc * n * kM));
+    }
+  } else {
+    for (int i = tid; i < nvalid * kM; i += THREADS) cp_async8(&sh.u[i], io.v_old + c0 * kM + i);
+  }
+  if (tid < (nvalid + 1) * n) face_traces<N>(P, io, c0, tid, a, b);
+}
+
+// One tile of the interface flux + update (+ lambda_max) of one solve.
 template <int N, int C = 64>
 __device__ __forceinline__ void face_tile(const FaceParams& P, const FaceIO& io,
                                           const StepParams& sp, long long tile, double dt,
-                                          FaceShared<N, C>& sh) {
+                                          FaceShared<N, C>& sh, double (&a)[kM],
+                                          double (&b)[kM]) {
   constexpr int n = N + 1, THREADS = FaceCfg<N, C>::THREADS;
   const double lam = dt * sp.inv_dx;
-  const long long c0 = tile * C;
-  const int nvalid = (int)((io.ncells - c0) < C ? (io.ncells - c0) : C);
-  const int stride = (P.dg ? 9 : 6) * n;
+  const long long c0 = tile * FaceCfg<N, C>::CELLS;
+  const int nvalid = face_valid<N, C>(io, tile);
   const int tid = threadIdx.x;
 
   // Rusanov flux at every tau node of faces c0-1/2 ... c0+nvalid-1/2
   for (int item = tid; item < (nvalid + 1) * n; item += THREADS) {
     const int f = item / n, l0 = item - f * n;
-    const long long cl = wrap_cell(c0 + f - 1, io.ncells), cr = wrap_cell(c0 + f, io.ncells);
-    const double* ta = io.trace + cl * stride + l0 * kM;          // qR of the left cell
-    const double* tb = io.trace + cr * stride + n * kM + l0 * kM; // qL of the right cell
-    double a[kM], b[kM], G2[kM];
-#pragma unroll
-    for (int r = 0; r < kM; ++r) {
-      a[r] = ta[r];
-      b[r] = tb[r];
-    }
+    double G2[kM];
+    if (item != tid) face_traces<N>(P, io, c0, item, a, b);
     if (P.bc == kBcOutflow && (c0 + f == 0 || c0 + f == io.ncells)) {
       // free outflow: the ghost side holds the boundary cell's mean of u^n
       const long long cb = c0 + f == 0 ? 0 : io.ncells - 1;
@@ -1199,12 +1240,13 @@ __device__ __forceinline__ void face_tile(const FaceParams& P, const FaceIO& io,
     for (int l0 = 0; l0 < n; ++l0) s = fma(sh.w[l0], sh.G[(f * n + l0) * kM + r], s);
     sh.Gs[f * kM + r] = hlam * s;
   }
+  cp_async_wait_all();
   __syncthreads();
   if (P.dg) {
     for (int item = tid; item < nvalid * n; item += THREADS) {
       const int lc = item / n, k = item - lc * n;
       const long long cell = c0 + lc;
-      const double* up = io.trace + cell * stride + 2 * n * kM + k * kM;
+      const double* up = sh.u + (lc * n + k) * kM;
       double* out = io.u_new + cell * (long long)(n * kM) + k * kM;
 #pragma unroll
       for (int r = 0; r < kM; ++r) {
@@ -1222,7 +1264,7 @@ __device__ __forceinline__ void face_tile(const FaceParams& P, const FaceIO& io,
     for (int item = tid; item < nvalid * kM; item += THREADS) {
       const int lc = item / kM, r = item - lc * kM;
       const long long cell = c0 + lc;
-      const double vn = io.v_old[cell * kM + r] - (sh.Gs[(lc + 1) * kM + r] - sh.Gs[lc * kM + r]);
+      const double vn = sh.u[lc * kM + r] - (sh.Gs[(lc + 1) * kM + r] - sh.Gs[lc * kM + r]);
       io.u_new[cell * kM + r] = vn;
       sh.u[lc * kM + r] = vn;
       const ff vf = d2ff(vn);
@@ -1249,26 +1291,34 @@ __device__ __forceinline__ void face_stage_tables(const FaceParams& P, FaceShare
     sh.psi0w[threadIdx.x] = P.ops.psi0[threadIdx.x] * P.ops.rw[threadIdx.x];
     sh.psi1w[threadIdx.x] = P.ops.psi1[threadIdx.x] * P.ops.rw[threadIdx.x];
   }
-  __syncthreads();
 }
 
 template <int N, int C>
 __device__ __forceinline__ void face_update_block(const FaceParams& P, FaceShared<N, C>& sh) {
-  double dt;
-  int last;
-  if (!corrector_step_dt(P.sp, &dt, &last)) return;
-  face_stage_tables<N, C>(P, sh);
   const FaceIO io{P.trace, P.v_old, P.u_new, P.ncells};
-  face_tile<N, C>(P, io, P.sp, blockIdx.x, dt, sh);
+  double dt, a[kM], b[kM];
+  int last;
+  face_prefetch<N, C>(P, io, blockIdx.x, sh, a, b);
+  face_stage_tables<N, C>(P, sh);
+  if (!corrector_step_dt(P.sp, &dt, &last)) {
+    cp_async_wait_all();
+    return;
+  }
+  __syncthreads();
+  face_tile<N, C>(P, io, P.sp, blockIdx.x, dt, sh, a, b);
   corrector_finish(P.sp, dt, last, blockIdx.x == 0 && threadIdx.x == 0);
 }
 
-// 4 resident blocks (64 registers): the fixed-point flux alone would take 71-74 (3
-// blocks), and the short phases between barriers want warps to fill them.  3 / 4 / 5
-// blocks: N = 3, 1e5 cells 45.4 / 41.9 / 45.6 us, N = 4, 1e6 cells 387 / 358 / 380,
-// N = 5, 1e5 cells 50.9 / 47.6 / 54.4, N = 7, 1e6 cells 485 / 426 / 450.
+// What bounds it: memory latency and barriers at the start of short blocks, then the
+// fixed-point flux (issue slots 40-60 %); DRAM 0.8-1.4 TB/s.  So the tile's C n flux
+// items fill whole passes of the block (64 cells gave 65 n items: a second pass with
+// one warp busy), and its memory is asked for before the step protocol is read.
+// 256-thread blocks of 64 cells -> this: WENO N = 4, 1e6 cells 322 -> 238 us, DG N = 2, 1e6
+// cells 328 -> 273, N = 5, 1e5 cells 48.1 -> 43.4, N = 7, 1e6 cells 426 -> 408.  Resident
+// threads 896 / 1024 / 1280: N = 4 236 / 238 / 256, N = 5 45.5 / 43.4 / 44.8, N = 7 432 /
+// 408 / 434 us.
 template <int N, int C = 64>
-__global__ void __launch_bounds__(FaceCfg<N, C>::THREADS, 4)
+__global__ void __launch_bounds__(FaceCfg<N, C>::THREADS, (FaceCfg<N, C>::MIN_BLOCKS))
     face_update_kernel(const __grid_constant__ FaceParams P) {
   __shared__ FaceShared<N, C> sh;
   face_update_block<N, C>(P, sh);
@@ -1280,6 +1330,7 @@ __global__ void __launch_bounds__(FaceCfg<N, C>::THREADS)
     face_update_multi_kernel(const __grid_constant__ FaceParams P, const MultiArgs M) {
   __shared__ FaceShared<N, C> sh;
   face_stage_tables<N, C>(P, sh);
+  __syncthreads();
   for (long long it = blockIdx.x; it < M.nitems; it += gridDim.x) {
     const TileItem item = M.items[it];
     const SlotDesc& d = M.slots[item.slot];
@@ -1290,7 +1341,9 @@ __global__ void __launch_bounds__(FaceCfg<N, C>::THREADS)
     int last;
     if (!corrector_step_dt(sp, &dt, &last)) continue;  // uniform over the block
     const FaceIO io{d.trace, d.u[par], const_cast<double*>(d.u[par ^ 1]), d.ncells};
-    face_tile<N, C>(P, io, sp, item.tile, dt, sh);
+    double a[kM], b[kM];
+    face_prefetch<N, C>(P, io, item.tile, sh, a, b);
+    face_tile<N, C>(P, io, sp, item.tile, dt, sh, a, b);
     corrector_finish(sp, dt, last, item.tile == 0 && threadIdx.x == 0);
   }
 }

@@ -265,7 +265,7 @@ ader_status rebuild(ader_server* srv) {
     for (size_t s = 0; s < srv->slots.size(); ++s) {
       const Req* r = srv->slots[s].req;
       if (!r || r->degree != N) continue;
-      const long long T = kServerFaceCells;
+      const long long T = kServerFaceCells - 1;  // the cells between a tile's faces
       for (long long t = 0; t < (r->ncells + T - 1) / T; ++t) items.push_back({(int)s, (int)t});
     }
     L.face_n = (long long)items.size() - L.face_off;

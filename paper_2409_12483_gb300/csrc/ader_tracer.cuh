@@ -358,9 +358,10 @@ __global__ void __launch_bounds__(FaceCfg<N, C>::THREADS)
   int last;
   if (!corrector_step_dt(P.sp, &dt, &last)) return;
   face_stage_tables<N, C>(P, sh.base);
+  __syncthreads();
   const double lam = dt * P.sp.inv_dx;
-  const long long c0 = (long long)blockIdx.x * C;
-  const int nvalid = (int)((P.ncells - c0) < C ? (P.ncells - c0) : C);
+  const long long c0 = (long long)blockIdx.x * FaceCfg<N, C>::CELLS;
+  const int nvalid = face_valid<N, C>(FaceIO{nullptr, nullptr, nullptr, P.ncells}, blockIdx.x);
   const int tid = threadIdx.x;
   for (int item = tid; item < (nvalid + 1) * n; item += THREADS) {
     const int f = item / n, l0 = item - f * n;
