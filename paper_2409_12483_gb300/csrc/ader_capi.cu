@@ -418,6 +418,7 @@ ader_status enqueue_step3d(ader_ctx* ctx, const double* src, double* dst, const 
   f.ops = ctx->basis.d;
   for (int j = 0; j < kMaxNs; ++j)
     for (int k = 0; k < kMaxN; ++k) f.Pf[j][k] = (float)ctx->basis.d.P[j][k];
+  f.pabs3 = projection_growth(f.ops, 3);
   CK(do_face3d(ctx->N, f, ctx->stream));
   ctx->launches += 3;
   if (ev) CK(cudaEventRecordWithFlags(ev[3], ctx->stream, cudaEventRecordExternal));

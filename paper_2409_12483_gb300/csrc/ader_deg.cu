@@ -512,6 +512,7 @@ cudaError_t ADER_CAT(launch_cfl3d_, ADER_DEG)(const Cfl3DParams& p, cudaStream_t
         f.ops.P[j][k] = p.P[j][k];
         f.Pf[j][k] = p.Pf[j][k];
       }
+    f.pabs3 = projection_growth(f.ops, 3);
     using B = Upd3Cfg<D, 128>;
     using S = Upd3Cfg<D, 64>;
     if (B::CPB != S::CPB && !use_big_blocks(p.ncells, B::CPB))

@@ -901,29 +901,50 @@ struct Upd3Cfg {
   static constexpr int CPB = NNN >= T ? 1 : T / NNN;  // cells per block
   static constexpr int USED = CPB * NNN;
   static constexpr int THREADS = (USED + 31) / 32 * 32;  // whole warps for the reductions
-  // The screening of lambda_max projects in FP32 throughout for N <= 1; above
-  // that the two separable passes stay FP64 and only the last pass is screened.
-  // With the rigorous FP32 bounds the all-FP32 projection (per-candidate FP64
-  // re-evaluation, outer loop rolled) measured 15.2 / 13.1 / 9.0 ms per face +
-  // update pair at N = 2 / 3 / 4 (96^3, 64^3, 40^3 cells) against 15.4 / 11.5 /
-  // 6.0 ms with the FP64 passes.
-  static constexpr bool kScreenAll = N <= 1;
-  // dynamic shared memory: U [CPB][NNN][5] (FP64); T1 [CPB][n n][Ns][5] (along
-  // zeta) and T2 [CPB][n][Ns Ns][5] (along eta), FP32 or FP64 as above; the upper
-  // bounds of the subcell speeds LT [CPB][Ns^3] (FP32); with an FP32 T1 and T2,
-  // their sums of |P| |u| A1 and A2 (the error bound), shaped as T1 and T2
-  static constexpr size_t kTBytes = kScreenAll ? sizeof(float) : sizeof(double);
+  // dynamic shared memory: U [CPB][NNN][5] (FP64); the projections along zeta, T1
+  // [CPB][n n][Ns][5], and eta, T2 [CPB][n][Ns Ns][5], in FP64 (the first screen keeps U
+  // and the projections there in FP32: n <= Ns, so both fit); the upper bounds of the
+  // subcell speeds LT [CPB][Ns^3] (FP32)
   static constexpr size_t kSmemBytes =
       (size_t)CPB * NNN * kM3 * sizeof(double) +
-      (size_t)CPB * (n * n * Ns + n * Ns * Ns) * kM3 * kTBytes +
-      (size_t)CPB * Ns * Ns * Ns * sizeof(float) +
-      (kScreenAll ? (size_t)CPB * (n * n * Ns + n * Ns * Ns) * kM3 * sizeof(float) : 0);
+      (size_t)CPB * (n * n * Ns + n * Ns * Ns) * kM3 * sizeof(double) +
+      (size_t)CPB * Ns * Ns * Ns * sizeof(float);
 };
+
+// One direction of the FP32 projection: NI independent lines of n values, `stride` apart
+// within a line, to Ns values `stride` apart; a thread takes whole lines, so that the
+// coefficients are uniform.
+template <int N>
+__device__ __forceinline__ void upd3_project(const Face3DParams& P, const float* in, float* out,
+                                             int stride) {
+  constexpr int n = N + 1, Ns = 2 * N + 1;
+  float x[n];
+#pragma unroll
+  for (int k = 0; k < n; ++k) x[k] = in[k * stride];
+#pragma unroll
+  for (int j = 0; j < Ns; ++j) {
+    float acc = 0.f;
+#pragma unroll
+    for (int k = 0; k < n; ++k) acc = fmaf(P.Pf[j][k], x[k], acc);
+    out[j * stride] = acc;
+  }
+}
 
 // u^{n+1} = volume term - sum_d (psi~_{k_d} G_high - psi_{k_d} G_low) / w_{k_d}, one
 // thread per (cell, node), CPB cells per block; then (want_lambda) the block
 // projects its cells' new states onto the Ns^3 subcells one direction at a time
 // through shared memory and reduces max_d lambda_d / h_d into ctl->lam[par ^ 1].
+//
+// lambda_max in two screens.  (1) Three FP32 passes and bounds on every subcell's speed
+// in FP32: a block none of whose upper bounds reaches the cut shared by all blocks
+// (lambda_cut) is done.  (2) The others project along zeta and eta in FP64 and bound the
+// speeds from there (tighter by the two passes' roundings); the subcells that still
+// reach the cut are evaluated in FP64.  The subcell of the largest speed passes both, so
+// the result is the FP64 maximum over every subcell.
+// What bounds it: DRAM for the update (the record, the faces and the new state, 0.9 GB at
+// 48^3, N = 3), shared memory and FP32 issue for screen (1).  The separable FP64 passes for
+// every block (6160 FP64 FMA per cell at N = 3) made face + update 2.96 ms per step at 48^3,
+// N = 3, 1.12 at N = 2; now 1.68 and 0.75 (N = 4, 32^3: 0.99).
 template <int N, int TB = 128>
 __global__ void __launch_bounds__(Upd3Cfg<N, TB>::THREADS)
     update3d_kernel(const __grid_constant__ Face3DParams P) {
@@ -932,6 +953,14 @@ __global__ void __launch_bounds__(Upd3Cfg<N, TB>::THREADS)
   extern __shared__ __align__(16) double dsm[];
   auto U = reinterpret_cast<double(*)[NNN][kM3]>(dsm);
   __shared__ unsigned long long s_wmax[C::THREADS / 32];
+  __shared__ unsigned s_umax[kM3];
+  __shared__ float s_cut;
+  double* T1 = dsm + CPB * NNN * kM3;              // [CPB][n n][Ns][5]
+  double* T2 = T1 + CPB * n * n * Ns * kM3;        // [CPB][n][Ns Ns][5]
+  float* LT = reinterpret_cast<float*>(T2 + CPB * n * Ns * Ns * kM3);  // [CPB][Ns^3]
+  float* UF = reinterpret_cast<float*>(T1);        // the first screen's [CPB][NNN][5]
+  float* F1 = UF + CPB * NNN * kM3;                // [CPB][n n][Ns][5]
+  float* F2 = reinterpret_cast<float*>(T2);        // [CPB][n][Ns Ns][5]
   // CFL mode (u_cfl set): lambda_max of a given state by the same separable,
   // screened projection -- the first step's time step -- without the update
   const bool cfl_only = P.u_cfl != nullptr;
@@ -943,9 +972,11 @@ __global__ void __launch_bounds__(Upd3Cfg<N, TB>::THREADS)
   const long long cell = (long long)blockIdx.x * CPB + lc;
   const bool valid = tid < C::USED && cell < P.ncells;
   const OpsD& o = P.ops;
+  if (tid < kM3) s_umax[tid] = 0u;
+  double un[kM3] = {1.0, 0.0, 0.0, 0.0, 1.0};
   if (valid && cfl_only) {
 #pragma unroll
-    for (int r = 0; r < kM3; ++r) U[lc][k][r] = P.u_cfl[(cell * NNN + k) * kM3 + r];
+    for (int r = 0; r < kM3; ++r) un[r] = P.u_cfl[(cell * NNN + k) * kM3 + r];
   } else if (valid) {
     const int k1 = k / (n * n), k2 = (k / n) % n, k3 = k % n;
     const long long plane = P.nx * P.ny;
@@ -957,107 +988,128 @@ __global__ void __launch_bounds__(Upd3Cfg<N, TB>::THREADS)
     const int tr[3] = {k2 * n + k3, k1 * n + k3, k1 * n + k2};  // transverse pair per direction
     const double* vol = P.trace + cell * REC + 6 * NNN * kM3 + k * kM3;
 #pragma unroll
-    for (int r = 0; r < kM3; ++r) {
-      double val = vol[r];
+    for (int r = 0; r < kM3; ++r) un[r] = vol[r];
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const double gh = P.gface[((hi[d] * 3 + d) * n * n + tr[d]) * kM3 + r];
-        const double gl = P.gface[((cell * 3 + d) * n * n + tr[d]) * kM3 + r];
-        val = fma(-fma(o.psi1[kd[d]], gh, -o.psi0[kd[d]] * gl), o.rw[kd[d]], val);
-      }
-      P.u_new[(cell * NNN + k) * kM3 + r] = val;
-      U[lc][k][r] = val;
+    for (int d = 0; d < 3; ++d) {
+      const double ch = -o.psi1[kd[d]] * o.rw[kd[d]], cl = o.psi0[kd[d]] * o.rw[kd[d]];
+      const double* gh = P.gface + ((hi[d] * 3 + d) * n * n + tr[d]) * kM3;
+      const double* gl = P.gface + ((cell * 3 + d) * n * n + tr[d]) * kM3;
+#pragma unroll
+      for (int r = 0; r < kM3; ++r) un[r] = fma(ch, gh[r], fma(cl, gl[r], un[r]));
     }
+#pragma unroll
+    for (int r = 0; r < kM3; ++r) P.u_new[(cell * NNN + k) * kM3 + r] = un[r];
   }
   if (!cfl_only && blockIdx.x == 0 && tid == 0) corrector_finish(P.sp, dt, last, true);
   if (!cfl_only && !P.want_lambda) return;  // uniform
-  __syncthreads();
-  // lambda_max of u_new over the Ns^3 subcells, screened as in the 1D interface
-  // kernel: bounds on the wave speeds of every subcell in FP32 (FP32 pipes),
-  // then FP64 only for the subcells whose upper bound reaches the block's
-  // largest lower bound, so the result is the FP64 maximum over every subcell.
-  // N <= 1 projects in FP32 throughout (three passes: the FP32 subcell average
-  // is within (3n + 8) 2^-24 sum |P| |P| |P| |u| of the exact one) and
-  // re-evaluates a candidate from u_new; above that the separable passes T1
-  // (zeta) and T2 (eta) stay FP64 and the screen covers the last (xi) pass
-  // (within (n + 4) 2^-24 sum |P| |T2|) and the speeds.
-  __shared__ float s_cut;
+  unsigned long long* slot = &P.sp.ctl->lam[cfl_only ? P.cfl_slot : P.sp.par ^ 1];
   const long long c0 = (long long)blockIdx.x * CPB;
+  const int ncells = (int)(P.ncells - c0 < CPB ? P.ncells - c0 : CPB);
   const float gf = (float)P.gamma, gm1f = (float)P.gm1;
   const float ih[3] = {(float)P.sp.inv_dx, (float)P.inv_dy, (float)P.inv_dz};
-  constexpr bool kAll = C::kScreenAll;
-  using TT = typename std::conditional<kAll, float, double>::type;
-  TT* T1 = reinterpret_cast<TT*>(dsm + CPB * NNN * kM3);  // [CPB][n n][Ns][5]
-  TT* T2 = T1 + CPB * n * n * Ns * kM3;                    // [CPB][n][Ns Ns][5]
-  float* LT = reinterpret_cast<float*>(T2 + CPB * n * Ns * Ns * kM3);  // [CPB][Ns^3]
-  float* A1 = LT + CPB * Ns * Ns * Ns;    // kAll: [CPB][n n][Ns][5]
-  float* A2 = A1 + CPB * n * n * Ns * kM3;  // kAll: [CPB][n][Ns Ns][5]
-  for (int it = tid; it < CPB * n * n * Ns; it += C::THREADS) {
-    const int c = it / (n * n * Ns), rem = it - c * n * n * Ns, kk = rem / Ns, j3 = rem - kk * Ns;
-    if (c0 + c >= P.ncells) continue;
+  __syncthreads();  // s_umax
+  {
+    unsigned m[kM3];
 #pragma unroll
     for (int r = 0; r < kM3; ++r) {
-      TT acc = TT(0);
-      float aab = 0.f;
-#pragma unroll
-      for (int k3 = 0; k3 < n; ++k3) {
-        if constexpr (kAll) {
-          const float x = d2f_trunc(U[c][kk * n + k3][r]);
-          acc = fmaf(P.Pf[j3][k3], x, acc);
-          aab = fmaf(fabsf(P.Pf[j3][k3]), fabsf(x), aab);
-        } else {
-          acc = fma(o.P[j3][k3], U[c][kk * n + k3][r], acc);
-        }
+      const float x = d2f_trunc(un[r]);
+      m[r] = valid ? __float_as_uint(fabsf(x)) : 0u;
+      if (valid) {
+        U[lc][k][r] = un[r];
+        UF[(lc * NNN + k) * kM3 + r] = x;
       }
-      T1[((c * n * n + kk) * Ns + j3) * kM3 + r] = acc;
-      if constexpr (kAll) A1[((c * n * n + kk) * Ns + j3) * kM3 + r] = aab;
+    }
+#pragma unroll
+    for (int r = 0; r < kM3; ++r) {
+      m[r] = __reduce_max_sync(0xffffffffu, m[r]);
+      if ((tid & 31) == 0) atomicMax(&s_umax[r], m[r]);
     }
   }
   __syncthreads();
-  for (int it = tid; it < CPB * n * Ns * Ns; it += C::THREADS) {
-    const int c = it / (n * Ns * Ns), rem = it - c * n * Ns * Ns, k1 = rem / (Ns * Ns),
-              jj = rem - k1 * Ns * Ns, j2 = jj / Ns, j3 = jj - j2 * Ns;
-    if (c0 + c >= P.ncells) continue;
+  // (1) zeta, eta, xi in FP32: the subcell average is within (3n + 8) 2^-24 sum |P||P||P||u|
+  // of the exact one, at most max |u| over the block times the cube of max_j sum_k |P_jk|
+  for (int it = tid; it < ncells * n * n * kM3; it += C::THREADS) {
+    const int line = it / kM3, r = it - line * kM3;  // line: (cell, k1, k2)
+    upd3_project<N>(P, UF + line * n * kM3 + r, F1 + line * Ns * kM3 + r, kM3);
+  }
+  __syncthreads();
+  for (int it = tid; it < ncells * n * Ns * kM3; it += C::THREADS) {
+    const int line = it / (Ns * kM3), q = it - line * Ns * kM3;  // line: (cell, k1); q: (j3, r)
+    upd3_project<N>(P, F1 + line * n * Ns * kM3 + q, F2 + line * Ns * Ns * kM3 + q, Ns * kM3);
+  }
+  __syncthreads();
+  float e1[kM3], lo_loc = 0.f, hi_loc = 0.f;
+  {
+    constexpr float eproj = (float)(3 * n + 8) * 0x1p-24f;
+#pragma unroll
+    for (int r = 0; r < kM3; ++r)
+      e1[r] = fmaf(eproj * P.pabs3, __uint_as_float(s_umax[r]), 0x1p-100f);
+  }
+  for (int it = tid; it < ncells * Ns * Ns; it += C::THREADS) {
+    const int c = it / (Ns * Ns), jj = it - c * Ns * Ns;
+    const float* t2 = F2 + (c * n * Ns * Ns + jj) * kM3;
+    float x[n][kM3];
+#pragma unroll
+    for (int k1 = 0; k1 < n; ++k1)
+#pragma unroll
+      for (int r = 0; r < kM3; ++r) x[k1][r] = t2[k1 * Ns * Ns * kM3 + r];
+#pragma unroll 1
+    for (int j1 = 0; j1 < Ns; ++j1) {
+      float v[kM3], lo, hi;
+#pragma unroll
+      for (int r = 0; r < kM3; ++r) {
+        v[r] = 0.f;
+#pragma unroll
+        for (int k1 = 0; k1 < n; ++k1) v[r] = fmaf(P.Pf[j1][k1], x[k1][r], v[r]);
+      }
+      speed_bounds_f32<3>(v, e1, ih, gf, gm1f, lo, hi);
+      lo_loc = fmaxf(lo_loc, lo);
+      hi_loc = fmaxf(hi_loc, hi);
+    }
+  }
+  unsigned long long fm = block_max_bits((unsigned long long)__float_as_uint(lo_loc), s_wmax);
+  if (tid == 0) s_cut = lambda_cut(slot, __uint_as_float((unsigned)fm));
+  __syncthreads();
+  if (!__syncthreads_or(hi_loc >= s_cut)) return;  // another block holds the maximum
+  // (2) T1 (zeta) and T2 (eta) in FP64; the last pass and the speeds in FP32, within
+  // (n + 4) 2^-24 sum |P| |T2|
+  for (int it = tid; it < ncells * n * n * Ns; it += C::THREADS) {
+    const int line = it / Ns, j3 = it - line * Ns, c = line / (n * n), kk = line - c * n * n;
 #pragma unroll
     for (int r = 0; r < kM3; ++r) {
-      TT acc = TT(0);
-      float aab = 0.f;
+      double acc = 0.0;
 #pragma unroll
-      for (int k2 = 0; k2 < n; ++k2) {
-        const int i1 = ((c * n * n + k1 * n + k2) * Ns + j3) * kM3 + r;
-        if constexpr (kAll) {
-          acc = fmaf(P.Pf[j2][k2], T1[i1], acc);
-          aab = fmaf(fabsf(P.Pf[j2][k2]), A1[i1], aab);
-        } else {
-          acc = fma(o.P[j2][k2], T1[i1], acc);
-        }
-      }
-      T2[((c * n + k1) * Ns * Ns + jj) * kM3 + r] = acc;
-      if constexpr (kAll) A2[((c * n + k1) * Ns * Ns + jj) * kM3 + r] = aab;
+      for (int k3 = 0; k3 < n; ++k3) acc = fma(o.P[j3][k3], U[c][kk * n + k3][r], acc);
+      T1[it * kM3 + r] = acc;
     }
   }
   __syncthreads();
-  constexpr float eproj = (float)(kAll ? 3 * n + 8 : n + 4) * 0x1p-24f;
-  float lo_loc = 0.f;
-  for (int it = tid; it < CPB * Ns * Ns * Ns; it += C::THREADS) {
+  for (int it = tid; it < ncells * n * Ns * Ns; it += C::THREADS) {
+    const int line = it / (Ns * Ns), jj = it - line * Ns * Ns, j2 = jj / Ns, j3 = jj - j2 * Ns;
+#pragma unroll
+    for (int r = 0; r < kM3; ++r) {
+      double acc = 0.0;
+#pragma unroll
+      for (int k2 = 0; k2 < n; ++k2)
+        acc = fma(o.P[j2][k2], T1[((line * n + k2) * Ns + j3) * kM3 + r], acc);
+      T2[it * kM3 + r] = acc;
+    }
+  }
+  __syncthreads();
+  constexpr float eproj = (float)(n + 4) * 0x1p-24f;
+  lo_loc = 0.f;
+  for (int it = tid; it < ncells * Ns * Ns * Ns; it += C::THREADS) {
     const int c = it / (Ns * Ns * Ns), rem = it - c * Ns * Ns * Ns, j1 = rem / (Ns * Ns),
               jj = rem - j1 * Ns * Ns;
-    if (c0 + c >= P.ncells) continue;
     float v[kM3], e[kM3];
 #pragma unroll
     for (int r = 0; r < kM3; ++r) {
       float acc = 0.f, aab = 0.f;
 #pragma unroll
       for (int k1 = 0; k1 < n; ++k1) {
-        const int i2 = ((c * n + k1) * Ns * Ns + jj) * kM3 + r;
-        if constexpr (kAll) {
-          acc = fmaf(P.Pf[j1][k1], T2[i2], acc);
-          aab = fmaf(fabsf(P.Pf[j1][k1]), A2[i2], aab);
-        } else {
-          const float t = d2f_trunc(T2[i2]);
-          acc = fmaf(P.Pf[j1][k1], t, acc);
-          aab = fmaf(fabsf(P.Pf[j1][k1]), fabsf(t), aab);
-        }
+        const float t = d2f_trunc(T2[((c * n + k1) * Ns * Ns + jj) * kM3 + r]);
+        acc = fmaf(P.Pf[j1][k1], t, acc);
+        aab = fmaf(fabsf(P.Pf[j1][k1]), fabsf(t), aab);
       }
       v[r] = acc;
       e[r] = fmaf(eproj, aab, 0x1p-100f);  // + the truncation of values below 2^-126
@@ -1066,40 +1118,23 @@ __global__ void __launch_bounds__(Upd3Cfg<N, TB>::THREADS)
     speed_bounds_f32<3>(v, e, ih, gf, gm1f, lo, LT[it]);
     lo_loc = fmaxf(lo_loc, lo);
   }
-  const unsigned long long fm = block_max_bits((unsigned long long)__float_as_uint(lo_loc), s_wmax);
-  if (tid == 0)
-    s_cut = lambda_cut(&P.sp.ctl->lam[cfl_only ? P.cfl_slot : P.sp.par ^ 1],
-                       __uint_as_float((unsigned)fm));
+  fm = block_max_bits((unsigned long long)__float_as_uint(lo_loc), s_wmax);
+  if (tid == 0) s_cut = lambda_cut(slot, __uint_as_float((unsigned)fm));
   __syncthreads();
   const float cut = s_cut;
   double lmax = 0.0;
   bool bad = false;
-  for (int it = tid; it < CPB * Ns * Ns * Ns; it += C::THREADS) {
+  for (int it = tid; it < ncells * Ns * Ns * Ns; it += C::THREADS) {
+    if (!(LT[it] >= cut)) continue;
     const int c = it / (Ns * Ns * Ns), rem = it - c * Ns * Ns * Ns, j1 = rem / (Ns * Ns),
-              jj = rem - j1 * Ns * Ns, j2 = jj / Ns, j3 = jj - j2 * Ns;
-    if (c0 + c >= P.ncells || !(LT[it] >= cut)) continue;
-    // the subcell average in FP64 by the separable sums (zeta, eta, then xi)
+              jj = rem - j1 * Ns * Ns;
     double v[kM3];
 #pragma unroll
     for (int r = 0; r < kM3; ++r) {
       double acc = 0.0;
 #pragma unroll
-      for (int k1 = 0; k1 < n; ++k1) {
-        double t2;
-        if constexpr (kAll) {
-          t2 = 0.0;
-#pragma unroll
-          for (int k2 = 0; k2 < n; ++k2) {
-            double t1 = 0.0;
-#pragma unroll
-            for (int k3 = 0; k3 < n; ++k3) t1 = fma(o.P[j3][k3], U[c][(k1 * n + k2) * n + k3][r], t1);
-            t2 = fma(o.P[j2][k2], t1, t2);
-          }
-        } else {
-          t2 = T2[((c * n + k1) * Ns * Ns + jj) * kM3 + r];
-        }
-        acc = fma(o.P[j1][k1], t2, acc);
-      }
+      for (int k1 = 0; k1 < n; ++k1)
+        acc = fma(o.P[j1][k1], T2[((c * n + k1) * Ns * Ns + jj) * kM3 + r], acc);
       v[r] = acc;
     }
     const double inv = rcp64(v[0]);
@@ -1115,7 +1150,7 @@ __global__ void __launch_bounds__(Upd3Cfg<N, TB>::THREADS)
     }
   }
   const unsigned long long bm = block_max_bits(dbits(lmax), s_wmax);
-  if (tid == 0) atomicMax(&P.sp.ctl->lam[cfl_only ? P.cfl_slot : (P.sp.par ^ 1)], bm);
+  if (tid == 0) atomicMax(slot, bm);
   if (bad) atomicOr(&P.sp.ctl->status, kStNonPhysical);
 }
 

@@ -224,6 +224,7 @@ struct Face3DParams {
   StepParams sp;
   OpsD ops;
   float Pf[kMaxNs][kMaxN];  // P in FP32 (the screening pass of lambda_max)
+  float pabs3;              // (max_j sum_k |P_jk|)^3, rounded up
 };
 
 struct Cfl3DParams {

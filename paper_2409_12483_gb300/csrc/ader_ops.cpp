@@ -3,6 +3,7 @@
 
 #include "ader_fix.h"
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -183,6 +184,17 @@ FxGas make_fx_gas(double gamma) {
   g.gl = h[1];
   g.gammaf = (float)gamma;
   return g;
+}
+
+float projection_growth(const OpsD& o, int d) {
+  double row = 0.0, p = 1.0 + 1e-6;
+  for (int j = 0; j < kMaxNs; ++j) {
+    double a = 0.0;
+    for (int k = 0; k < kMaxN; ++k) a += std::fabs(o.P[j][k]);
+    row = std::max(row, a);
+  }
+  for (int i = 0; i < d; ++i) p *= row;
+  return (float)p;
 }
 
 int build_basis(int N, bool weno, Basis* out) {

@@ -112,6 +112,9 @@ struct FxGas {
 // the same and gamma itself, for the interface kernels (ader_fixr.cuh)
 FxGas make_fx_gas(double gamma);
 
+// (max_j sum_k |P_jk|)^d rounded up: the growth of max |u| in d subcell projections
+float projection_growth(const OpsD& o, int d);
+
 // Returns 0 on success.  weno != 0 also builds the WENO tables (N even, 2 <= N).
 int build_basis(int N, bool weno, Basis* out);
 
