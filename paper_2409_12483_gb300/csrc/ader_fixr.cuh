@@ -129,7 +129,8 @@ __device__ __forceinline__ fxi fx_sound_speed(fxi rho, fxi p57, int r1, float c0
 }
 
 // Twice the Rusanov flux between a (low side) and b in direction DIR.  False: not taken
-// (G2 unset).  speed: s and the two normal velocities as doubles, where asked for.
+// (G2 unset).  speed, where asked for: s, the two normal velocities and the bound on the
+// relative error of s, for further variables' fluxes.
 template <int D, int DIR>
 __device__ __forceinline__ bool fx_rusanov2(const double* a, const double* b, double* G2,
                                             const FxGas& g, double* speed = nullptr) {
@@ -177,7 +178,7 @@ __device__ __forceinline__ bool fx_rusanov2(const double* a, const double* b, do
   jf *= 0x1p-61f;
   ff *= 0x1p-25f;
   fxi sd[M];
-  double s_out = 0.0;
+  double s_out = 0.0, s_err = 1e-6;
   if (sf * jf * 1e-6f <= 1e-16f * ff) {
     if (!(sf < 15.0f)) return false;
     const int si = __float2int_rn(sf * 0x1p27f);
@@ -206,6 +207,7 @@ __device__ __forceinline__ bool fx_rusanov2(const double* a, const double* b, do
       fx_mac(t, s.h, s.l, fx_split(r < M - 1 ? d[r] : d[r] * 8));
       sd[r] = r < M - 1 ? fx_fold<3>(t) : fx_fold<4>(t);
     }
+    s_err = 0x1p-45;
     if (speed) s_out = fx_to_double_int(sm, ec - 57);
   }
 #pragma unroll
@@ -217,6 +219,7 @@ __device__ __forceinline__ bool fx_rusanov2(const double* a, const double* b, do
     speed[0] = s_out;
     speed[1] = fx_to_double_int(((fxi)Ua.h << 32) + Ua.l, ec - 60);
     speed[2] = fx_to_double_int(((fxi)Ub.h << 32) + Ub.l, ec - 60);
+    speed[3] = s_err;
   }
   return true;
 }

@@ -52,6 +52,23 @@ __device__ __forceinline__ void rusanov2_nc(const double* a, const double* b, do
   *bt = ubar * (b[3] - a[3]);
 }
 
+// The same with the Euler part in fixed point (see fx_rusanov2_src).  The mean of u along
+// the segment is the mean of its ends up to (d rho / rho) d u: taken where that, times the
+// tracer jump, is below the rounding of s phi.
+__device__ __forceinline__ bool fx_rusanov2_nc(const double* a, const double* b, double* G2,
+                                               double* bt, const FxGas& g) {
+  double S[4];
+  if (!fx_rusanov2<1, 0>(a, b, G2, g, S)) return false;
+  const double d = b[3] - a[3];
+  if (!fx_speed_holds(a[3], b[3], d, S[3])) return false;
+  const float q = fmaxf(fabsf(d2f_trunc(a[3])), fabsf(d2f_trunc(b[3]))), s = d2f_trunc(S[0]);
+  const float bend = fabsf(d2f_trunc(b[0] - a[0])) * fabsf(d2f_trunc(S[2] - S[1]));
+  if (!(bend * fabsf(d2f_trunc(d)) <= 1e-16f * s * q * d2f_trunc(a[0]))) return false;
+  G2[3] = -S[0] * d;
+  *bt = 0.5 * (S[1] + S[2]) * d;
+  return true;
+}
+
 template <int N, int CPB_>
 struct NcCfg {
   static constexpr int n = N + 1;
@@ -374,7 +391,7 @@ __global__ void __launch_bounds__(FaceCfg<N, C>::THREADS)
       a[r] = ta[r];
       b[r] = tb[r];
     }
-    rusanov2_nc(a, b, G2, &bt, P.gamma, P.gm1);
+    if (!fx_rusanov2_nc(a, b, G2, &bt, P.gas)) rusanov2_nc(a, b, G2, &bt, P.gamma, P.gm1);
 #pragma unroll
     for (int r = 0; r < M; ++r) sh.G[(f * n + l0) * M + r] = G2[r];
     sh.B[f * n + l0] = bt;

@@ -86,3 +86,30 @@ def test_states(cuda, oracle_mod, D, N, kind):
 def test_adiabatic_index(cuda, oracle_mod, D, N, gamma):
     """gamma - 1 above 1 takes the FP64 form"""
     run(cuda, oracle_mod, D, N, lambda v: None, gamma=gamma)
+
+
+@pytest.mark.parametrize("system", ["reacting", "tracer"])
+@pytest.mark.parametrize("N", [1, 3, 5, 7])
+@pytest.mark.parametrize("what", ["all", "others", "none"])
+@pytest.mark.parametrize("jump", [1e-14, 1e-11, 1e-9, 1e-6, 1e-2, 10.0])
+def test_systems_jumps(cuda, oracle_mod, system, N, what, jump):
+    """jumps of the further variables alone (their own bound on the wave speed's error and
+    the path mean of u) and together with the Euler ones"""
+    import test_gpu_fixed_systems as fs
+    nc = 67
+    o = oracle_mod.ReactingOracle(N, omega=1.0) if system == "reacting" else oracle_mod.NCOracle(N)
+    u = (fs.reacting if system == "reacting" else fs.tracer)(o, nc, N)
+    g = np.random.default_rng(N)
+    f = (1.0 + jump) ** g.uniform(-1, 1, (4, nc, 1))
+    if what == "all":
+        u[..., 0] *= f[0]
+        u[..., 1] *= f[0] * np.sqrt(f[1])
+        u[..., 2] *= f[0] * f[1]
+    if what != "none":
+        for r in range(3, u.shape[-1]):
+            u[..., r] *= f[r - 1]
+    # (the wave speed is the Euler part's)
+    dt = 0.5 * oracle_mod.Oracle(N).dg_dt(np.ascontiguousarray(u[..., :3]), 1.0 / nc)
+    got, _ = fs.gpu_step(u, N, dt, system, **({"omega": 1.0} if system == "reacting" else {}))
+    step = o.dg_step if system == "reacting" else o.step
+    assert fs.worst(got, step(u, 1.0 / nc, dt)[0]) < 1e-12
