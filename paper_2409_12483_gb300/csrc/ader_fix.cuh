@@ -81,7 +81,6 @@ struct FixShared {
 
 // 2^k as a double, |k| < 1000
 __device__ __forceinline__ double fx_pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
-__device__ __forceinline__ float fx_pow2f(int k) { return __int_as_float((127 + k) << 23); }
 
 // x 2^k for a normal x (0 below), |k| < 200, on the integer pipe
 __device__ __forceinline__ double fx_scale(double x, int k) {

@@ -34,6 +34,17 @@ __device__ __forceinline__ fxi fx_from_double(double x, int e) {
   return hi < 0 ? -v : v;
 }
 
+// x in [0, 1] at frac 60, truncated
+__device__ __forceinline__ fxi fx_from_float(float x) {
+  const unsigned b = __float_as_uint(x);
+  const int ex = (int)(b >> 23);
+  const fxi m = ex ? (fxi)((b & 0x7fffffu) | 0x800000u) : 0;
+  return ex >= 90 ? m << (ex - 90) : m >> min(90 - ex, 63);
+}
+
+// 2^k as a float (|k| < 126)
+__device__ __forceinline__ float fx_pow2f(int k) { return __int_as_float((127 + k) << 23); }
+
 // X 2^k rounded to nearest, on the integer pipe (|k| < 500)
 __device__ __forceinline__ double fx_to_double_int(fxi x, int k) {
   const unsigned long long a = (unsigned long long)(x < 0 ? -x : x);

@@ -1454,21 +1454,18 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflPar
 // underflow of x^8), so a relative error rho_S of x_S moves r_S by at most
 // 8.1 (rho_min + rho_S) + 15 2^-24 and om_S by twice the largest of those plus
 // 6 2^-24.  With om_2 = 1 - om_0 - om_1 the change of the reconstruction is
-// sum_{S=0,1} dom_S (p_S - p_2), and |p_S - p_2| <= sum_j |d_S,j| on the cell
+// sum_{S=0,1} dom_S (p_S - p_2), and |p_S - p_2| <= D_S = sum_j |d_S,j| on the cell
 // (|t| <= 1).  Returns false (use FP64) when that bound is too large, when a
 // relative error exceeds 2^-12, or on any non-finite value.
 template <int N>
-__device__ __forceinline__ bool weno_weights_f32(const WenoOps& wo, const double (&a)[3][N + 1],
-                                                 const double (&d)[2][N + 1], double* om0,
-                                                 double* om1) {
+__device__ __forceinline__ bool weno_weights_f32(const WenoOps& wo, const float (&a)[3][N + 1],
+                                                 float D0, float D1, float* om0, float* om1) {
   constexpr int n = N + 1;
   constexpr float u = 0x1p-24f;
   float x[3], rho[3];
 #pragma unroll
   for (int S = 0; S < 3; ++S) {
-    float af[n];
-#pragma unroll
-    for (int j = 1; j < n; ++j) af[j] = d2f_trunc(a[S][j]);
+    const float(&af)[n] = a[S];
     float sig = 0.f, asig = 0.f;
 #pragma unroll
     for (int j = 1; j < n; ++j) {
@@ -1505,18 +1502,103 @@ __device__ __forceinline__ bool weno_weights_f32(const WenoOps& wo, const double
   const float w0 = nl0 / W, w1 = nl1 / W;
   // relative error of every om_S (om_2's included through om_0 + om_1)
   const float eom = 2.f * (8.1f * 2.f * rho_m + 15.f * u) + 6.f * u;
-  float D0 = 0.f, D1 = 0.f;
-#pragma unroll
-  for (int j = 0; j < n; ++j) {
-    D0 += fabsf(d2f_trunc(d[0][j]));
-    D1 += fabsf(d2f_trunc(d[1][j]));
-  }
   // the truncations and the sums (n terms) stay within (n + 2) 2^-24 of D_S
   const float dev = eom * (w0 * D0 + w1 * D1) * (1.f + (float)(n + 4) * u);
-  const float ref = 0x1p-52f * fabsf(d2f_trunc(a[2][0]));
+  const float ref = 0x1p-52f * fabsf(a[2][0]);
   if (!(dev <= ref) || !(W < 1e30f)) return false;
-  *om0 = f2d_bits(w0);
-  *om1 = f2d_bits(w1);
+  *om0 = w0;
+  *om1 = w1;
+  return true;
+}
+
+// The reconstruction of one variable in fixed point (arithmetic of ader_fix.h).
+//
+// What bounds it.  FP64: ~96 operations per cell and variable, 64 issue cycles of a
+// scheduler each (FP64 pipe 83 % busy).  Here the three polynomials and the nodal values
+// are ~240 wide integer multiply-adds of 4 cycles (N = 4, 1e6 cells: 569 -> 183 us; issue
+// slots 60 %, no FP64).  5 or 6 resident blocks asked of the registers (95): 396 and 377
+// against 382 us where some cells take the FP64 form, so no bound is given.
+//
+// Units: 2^e above the stencil's largest value.  Averages at frac 61; monomial
+// coefficients at frac F = 59 - fxs (row sums of |amono| below 2^fxs), off by 2^-(F + 1) of
+// the unit each -- an FP64 coefficient, a sum of products of the same size, by 2^-53 of
+// that size per term; nodal values at F.  Weights as in the FP64 form's FP32 screen, at
+// frac 60.  False, and nothing written, where the values of the stencil differ by more
+// than a factor 4 to 8 (a common unit would cost the small ones digits), the unit is
+// outside 2^+-30, or FP32 weights will not do: the FP64 form then runs.
+constexpr int kFxWenoMax = 4;  // degree: the 64-bit sums have room for N + 1 <= 5 terms
+
+// x 2^k as a float within 2^-24 (one conversion on the quarter-rate pipe)
+__device__ __forceinline__ float fx_to_float(fxi x, int k) {
+  return __ll2float_rn(x) * fx_pow2f(k);
+}
+
+template <int N>
+__device__ __forceinline__ bool weno_fix(const WenoOps& wo, const double* vs, double* out) {
+  constexpr int n = N + 1, h = N / 2;
+  int fmax_ = 0, fmin_ = 0x7ff;
+#pragma unroll
+  for (int s = 0; s <= 2 * N; ++s) {
+    const int f = (__double2hiint(vs[s]) >> 20) & 0x7ff;
+    fmax_ = max(fmax_, f);
+    fmin_ = min(fmin_, f);
+  }
+  const int e = fmax_ ? fmax_ - 1022 : 0, F = 59 - wo.fxs;
+  if (wo.fxs < 0 || abs(e) > 30 || fmin_ < fmax_ - 2) return false;
+  fxi a[3][n];
+  {
+    Fx2 x[2 * N + 1];
+#pragma unroll
+    for (int s = 0; s <= 2 * N; ++s) x[s] = fx_split(fx_from_double(vs[s], e));
+#pragma unroll
+    for (int S = 0; S < 3; ++S) {
+      const int base = S == 0 ? h : S == 1 ? 0 : N;
+#pragma unroll
+      for (int j = 0; j < n; ++j) {
+        FxAcc t = fx_zero<0>();
+#pragma unroll
+        for (int k = 0; k < n; ++k)
+          fx_mac(t, wo.amonox[S][j][k][0], wo.amonox[S][j][k][1], x[base + k]);
+        a[S][j] = fx_fold<0>(t);
+      }
+    }
+  }
+  float af[3][n], D[2] = {0.f, 0.f}, w0, w1;
+#pragma unroll
+  for (int j = 0; j < n; ++j) {
+#pragma unroll
+    for (int S = 0; S < 3; ++S) af[S][j] = j || S == 2 ? fx_to_float(a[S][j], e - F) : 0.f;
+#pragma unroll
+    for (int S = 0; S < 2; ++S) {
+      a[S][j] -= a[2][j];
+      D[S] += fabsf(fx_to_float(a[S][j], e - F));
+    }
+  }
+  if (!weno_weights_f32<N>(wo, af, D[0], D[1], &w0, &w1)) return false;
+  Fx2 om[2], ah[n];
+  om[0] = fx_split(fx_from_float(w0));
+  om[1] = fx_split(fx_from_float(w1));
+  fxi ah0 = 0;
+#pragma unroll
+  for (int j = 0; j < n; ++j) {
+    FxAcc t = fx_zero<4>();
+    fx_mac(t, om[0].h, om[0].l, fx_split(a[0][j]));
+    fx_mac(t, om[1].h, om[1].l, fx_split(a[1][j]));
+    const fxi x = a[2][j] + fx_fold<4>(t);
+    ah[j] = fx_split(x);
+    if (j == 0) ah0 = x;
+  }
+#pragma unroll
+  for (int q = 0; q < h; ++q) {
+    FxAcc ev = fx_zero<3>(), od = fx_zero<3>();
+#pragma unroll
+    for (int j = 1; j < n; ++j)
+      fx_mac((j & 1) ? od : ev, wo.vnodx[q][j][0], wo.vnodx[q][j][1], ah[j]);
+    const fxi E = ah0 + fx_fold<3>(ev), O = fx_fold<3>(od);
+    out[q * kM] = fx_to_double_int(E + O, e - F);
+    out[(N - q) * kM] = fx_to_double_int(E - O, e - F);
+  }
+  out[h * kM] = fx_to_double_int(ah0, e - F);
   return true;
 }
 
@@ -1532,7 +1614,8 @@ static __device__ __noinline__ Weights3 weno_weights_slow(double l0, double l1, 
   return Weights3{t0 / ws, t1 / ws, t2 / ws};
 }
 
-// One thread per cell and conserved variable loop.  Each candidate polynomial
+// One thread per cell, a loop over the variables: weno_fix, or where that is not taken, in
+// FP64 as follows.  Each candidate polynomial
 // is formed in monomial coefficients a_j (t = 2 xi - 1) directly from its N+1
 // cell averages (amono = mono * ainv, built in long double); sigma uses only
 // the non-zero entries of smono (j + l even); the normalised weights
@@ -1559,6 +1642,10 @@ __global__ void __launch_bounds__(128) weno_kernel(const __grid_constant__ WenoP
         j = wrap_cell(j, nc);
       }
       vs[s + N] = P.v[j * kM + r];
+    }
+    double* out = P.w + i * (n * kM) + r;
+    if constexpr (N <= kFxWenoMax) {
+      if (weno_fix<N>(P.wo, vs, out)) continue;
     }
     double a[3][n];
     {
@@ -1600,7 +1687,18 @@ __global__ void __launch_bounds__(128) weno_kernel(const __grid_constant__ WenoP
 #pragma unroll
       for (int j = 0; j < n; ++j) d[S][j] = a[S][j] - a[2][j];
     double om0, om1;
-    if (!weno_weights_f32<N>(P.wo, a, d, &om0, &om1)) {
+    float af[3][n], D[2] = {0.f, 0.f}, w0, w1;
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+#pragma unroll
+      for (int S = 0; S < 3; ++S) af[S][j] = d2f_trunc(a[S][j]);
+#pragma unroll
+      for (int S = 0; S < 2; ++S) D[S] += fabsf(d2f_trunc(d[S][j]));
+    }
+    if (weno_weights_f32<N>(P.wo, af, D[0], D[1], &w0, &w1)) {
+      om0 = f2d_bits(w0);
+      om1 = f2d_bits(w1);
+    } else {
       // FP64 weights where the FP32 ones cannot be shown to be exact enough
       double x8[3];
 #pragma unroll
@@ -1636,7 +1734,6 @@ __global__ void __launch_bounds__(128) weno_kernel(const __grid_constant__ WenoP
     for (int j = 0; j < n; ++j) ah[j] = fma(om0, d[0][j], fma(om1, d[1][j], a[2][j]));
     // nodal values at the GL nodes, symmetric about the cell centre
     // (t_{N-q} = -t_q, t_{N/2} = 0): even and odd parts of the polynomial
-    double* out = P.w + i * (n * kM) + r;
 #pragma unroll
     for (int q = 0; q < N / 2; ++q) {
       double ev = ah[0], od = 0.0;

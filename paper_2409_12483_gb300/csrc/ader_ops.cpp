@@ -347,6 +347,7 @@ int build_basis(int N, bool weno, Basis* out) {
         for (int j = 0; j < n; ++j) {
           V[q][j] = p;
           wo.vnod[q][j] = (double)p;
+          split_fx(p, 61, wo.vnodx[q][j]);
           p *= tq;
           Mono[q][j] = (q == j);
         }
@@ -355,6 +356,7 @@ int build_basis(int N, bool weno, Basis* out) {
       for (int j = 0; j < n; ++j)
         for (int k = 0; k < n; ++k) wo.mono[j][k] = (double)Mono[j][k];
     }
+    ld amono[3][kMaxN][kMaxN], row_max = 0;
     for (int S = 0; S < 3; ++S) {
       ld A[kMaxN][kMaxN], I[kMaxN][kMaxN];
       for (int j = 0; j < n; ++j)
@@ -374,9 +376,21 @@ int build_basis(int N, bool weno, Basis* out) {
           wo.ainv[S][j][k] = (double)I[j][k];
           ld a = 0;  // mono * ainv[S] in long double
           for (int m = 0; m < n; ++m) a += Mono[j][m] * I[m][k];
+          amono[S][j][k] = a;
           wo.amono[S][j][k] = (double)a;
         }
+      for (int j = 0; j < n; ++j) {
+        ld row = 0;
+        for (int k = 0; k < n; ++k) row += fabsl(amono[S][j][k]);
+        row_max = std::max(row_max, row);
+      }
     }
+    wo.fxs = 0;
+    while (ldexpl(1.0L, wo.fxs) < row_max) ++wo.fxs;
+    if (wo.fxs > 8) wo.fxs = -1;
+    for (int S = 0; S < 3 && wo.fxs >= 0; ++S)
+      for (int j = 0; j < n; ++j)
+        for (int k = 0; k < n; ++k) split_fx(amono[S][j][k], 62 - wo.fxs, wo.amonox[S][j][k]);
     // sigma = sum_{a=1..N} int_0^1 (d^a p / d xi^a)^2 d xi, p = sum_j a_j t^j:
     // d^a t^j / d xi^a = 2^a j!/(j-a)! t^(j-a);  int_0^1 d xi = 1/2 int_{-1}^{1} dt
     for (int j = 1; j < n; ++j)

@@ -82,6 +82,9 @@ struct WenoOps {
   double vnod[kMaxN][kMaxN];      // nodal values from monomial coefficients: c_q = sum_j vnod[q][j] a_j, t_q^j
   float smonof[kMaxN][kMaxN];     // smono, eps and lin rounded to FP32 (the screened weights)
   float epsf, linf[3];
+  // limbs for the fixed-point form (weno_fix): amono at frac 62 - fxs, vnod at frac 61;
+  // fxs: the row sums of |amono| are below 2^fxs (-1: no such form)
+  int amonox[3][kMaxN][kMaxN][2], vnodx[kMaxN][kMaxN][2], fxs;
 };
 
 struct Basis {
