@@ -1,9 +1,9 @@
 // ader_fix.h -- 60-bit fixed-point arithmetic on 32-bit integer multipliers, the
 // number form of the FP64 predictor's inner loop (ader_fix.cuh).
 //
-// GB300 issues 2 FP64 lanes per SM and clock against 64 lanes of 32 x 32 + 64-bit
-// integer multiply-add (mad.wide: 62.7 lanes measured), so a product of two
-// two-limb integers (3 mad.wide) costs a tenth of one DFMA.  Inside one cell the
+// GB300 issues 2 FP64 lanes per SM and clock against 32 lanes of 32 x 32 + 64-bit
+// integer multiply-add (mad.wide, measured on data that varies), so a product of two
+// two-limb integers (3 mad.wide) costs a fifth of one DFMA.  Inside one cell the
 // scheme's contractions mix all nodes, so the rounding of a result is set by the
 // largest value of the cell: a common exponent per cell and variable loses
 // nothing against a floating-point significand, and 57 fraction bits below that
