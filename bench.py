@@ -46,10 +46,10 @@ M = 3
 
 # DRAM traffic of the predictor kernel from an ncu capture, valid only for the
 # kernel sources whose hash is recorded with it (see profiles/).
-TRAFFIC_RECORD = {"sha256": "a37bbf3ccba3f2d0b9a3d334289287ce81dd4eda92acf8e0b9c5b1c58362351c",
-                  "bytes_per_launch": 14493525,
-                  "source": "profiles/launches_dg_n5_1e5cells.md (dram read 14.489 MB + write 0.005 MB "
-                            "per timed-region launch of this bench, mean of 3)"}
+TRAFFIC_RECORD = {"sha256": "6045189a4f509ebe29ecf35a3bca4eb1c9cad0a47a2c95a07863e985b50ad6b3",
+                  "bytes_per_launch": 15233000,
+                  "source": "profiles/fixed_point_kernels.md (dram read 14.470 MB + write 0.76-0.80 MB per "
+                            "launch of this state's time loop)"}
 
 
 def kernel_source_hash() -> str:
