@@ -46,7 +46,7 @@ M = 3
 
 # DRAM traffic of the predictor kernel from an ncu capture, valid only for the
 # kernel sources whose hash is recorded with it (see profiles/).
-TRAFFIC_RECORD = {"sha256": "6045189a4f509ebe29ecf35a3bca4eb1c9cad0a47a2c95a07863e985b50ad6b3",
+TRAFFIC_RECORD = {"sha256": "f9a5ae76c195ab7a1e3a02c49d9bb5074404afec4a6a5cc6a22eb627846c6e78",
                   "bytes_per_launch": 15233000,
                   "source": "profiles/fixed_point_kernels.md (dram read 14.470 MB + write 0.76-0.80 MB per "
                             "launch of this state's time loop)"}

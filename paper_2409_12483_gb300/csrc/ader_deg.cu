@@ -124,10 +124,10 @@ cudaError_t prepare_cpb() {
   }
 }
 
-// The FP64 form runs in fixed point (ader_fix.cuh) from N = 1, except for a given
-// q (from_q: only the epilogue) and an adiabatic index outside its tables; the
-// tuned cells per block choose its warps per block: 2, 4 or 8 for 16, 32 or 64.
-template <int CPB>
+// The FP64 form runs in fixed point (ader_fix.cuh) from N = 1, except for an adiabatic
+// index outside its tables; the tuned cells per block choose its warps per block: 2, 4 or
+// 8 for 16, 32 or 64.  Q: a given q, only the epilogue.
+template <int CPB, bool Q = false>
 cudaError_t launch_predict_fix(const PredictParams& p, cudaStream_t s) {
   using C = FixCfg<D, CPB / 8>;
   const long long blocks = (p.ncells + C::CELLS - 1) / C::CELLS;
@@ -135,16 +135,16 @@ cudaError_t launch_predict_fix(const PredictParams& p, cudaStream_t s) {
   // the blocks that fit at once; each takes every grid-th tile
   const long long resident = 152LL * C::MIN_BLOCKS;
   const long long grid = blocks < resident ? blocks : resident;
-  predict_fix_kernel<D, C::WPB><<<(unsigned)grid, C::THREADS, C::kSmemBytes, s>>>(p);
+  predict_fix_kernel<D, C::WPB, Q><<<(unsigned)grid, C::THREADS, C::kSmemBytes, s>>>(p);
   return cudaGetLastError();
 }
 
-template <int CPB>
+template <int CPB, bool Q = false>
 cudaError_t prepare_fix() {
   using C = FixCfg<D, CPB / 8>;
   if constexpr (!C::kValid) return cudaSuccess;
   else
-    return cudaFuncSetAttribute(predict_fix_kernel<D, C::WPB>,
+    return cudaFuncSetAttribute(predict_fix_kernel<D, C::WPB, Q>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes);
 }
 
@@ -180,7 +180,8 @@ cudaError_t launch_predict_cpb(const PredictParams& p, cudaStream_t s) {
     const long long blocks = (p.ncells + C::CPB - 1) / C::CPB;
     if (blocks <= 0 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     if constexpr (D >= 1) {
-      if (p.prec == 0 && !p.from_q && p.fix) return launch_predict_fix<CPB>(p, s);
+      if (p.from_q && p.fix) return launch_predict_fix<32, true>(p, s);
+      if (p.prec == 0 && p.fix) return launch_predict_fix<CPB>(p, s);
     }
     if (p.prec == 1 && !p.from_q)
       predict_kernel<D, 1, CPB><<<(unsigned)blocks, C::THREADS, C::kSmemBytes, s>>>(p);
@@ -325,6 +326,7 @@ cudaError_t ADER_CAT(prepare_degree_, ADER_DEG)() {
   cudaError_t e;
   if ((e = prepare_fix<16>()) != cudaSuccess) return e;
   if ((e = prepare_fix<32>()) != cudaSuccess) return e;
+  if ((e = prepare_fix<32, true>()) != cudaSuccess) return e;
   if ((e = prepare_fix<64>()) != cudaSuccess) return e;
   if ((e = prepare_cpb<16>()) != cudaSuccess) return e;
   if ((e = prepare_cpb<32>()) != cudaSuccess) return e;
