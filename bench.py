@@ -46,7 +46,7 @@ M = 3
 
 # DRAM traffic of the predictor kernel from an ncu capture, valid only for the
 # kernel sources whose hash is recorded with it (see profiles/).
-TRAFFIC_RECORD = {"sha256": "f9a5ae76c195ab7a1e3a02c49d9bb5074404afec4a6a5cc6a22eb627846c6e78",
+TRAFFIC_RECORD = {"sha256": "e7f6474525a6a668fa0ba5571c319f8b6bd2ed8499939e46dc9ec34a9d11feed",
                   "bytes_per_launch": 15233000,
                   "source": "profiles/fixed_point_kernels.md (dram read 14.470 MB + write 0.76-0.80 MB per "
                             "launch of this state's time loop)"}

@@ -164,8 +164,8 @@ struct FixStats {
 
 // The cells of one warp of a block's tile.  ke: the exponent the warp's kappa~ table
 // was built with (kFixNoTable at first).
-// Q: q is given (io.q_in) and only the epilogue runs; its maxima set the units.  (The
-// predictor / corrector pair of calls, N = 3, 20011 cells: 62 -> 55 us for both and a copy.)
+// Q: q is given (io.q_in) and only the epilogue runs; its maxima set the units
+// (ader_predict and ader_correct, N = 3, 20011 cells: 62 -> 55 us together).
 constexpr int kFixNoTable = 1 << 20;
 template <int N, int WPB, bool Q = false>
 __device__ __forceinline__ void predict_fix_warp(const PredictParams& P, const TileIO& io,
