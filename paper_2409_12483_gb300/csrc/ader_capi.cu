@@ -311,6 +311,7 @@ ader_status enqueue_limiter(ader_ctx* ctx, const double* src, double* dst, const
   l.s1 = ctx->sub1;
   l.gamma = ctx->opt.gamma;
   l.gm1 = ctx->opt.gamma - 1.0;
+  l.gas = make_fx_gas(l.gamma);
   l.delta0 = ctx->opt.nad_delta0;
   l.eps = ctx->opt.nad_eps;
   l.sp = sp;

@@ -1153,6 +1153,13 @@ __device__ __forceinline__ void rusanov2_screened(const double* a, const double*
   G2[2] = fma(-s, d2, F2);
 }
 
+// The flux of a face of the 1D Euler interface kernel.  The limiter takes it off again
+// where a subcell flux replaces it (lim_recompute_kernel), so it is formed here for both.
+__device__ __forceinline__ void face_flux2(const double* a, const double* b, double* G2,
+                                           double gamma, double gm1, const FxGas& gas) {
+  if (!fx_rusanov2<1, 0>(a, b, G2, gas)) rusanov2_screened(a, b, G2, gamma, gm1, (float)gamma);
+}
+
 // What a tile needs from memory, asked for before anything waits: each cell's u + volume
 // term (DG) or average (FV) by asynchronous copies into sh.u, the traces of the thread's
 // first (face, tau) item into a, b.
@@ -1225,8 +1232,7 @@ __device__ __forceinline__ void face_tile(const FaceParams& P, const FaceIO& io,
         g[r] = m;
       }
     }
-    if (!fx_rusanov2<1, 0>(a, b, G2, P.gas))
-      rusanov2_screened(a, b, G2, P.gamma, P.gm1, (float)P.gamma);
+    face_flux2(a, b, G2, P.gamma, P.gm1, P.gas);
 #pragma unroll
     for (int r = 0; r < kM; ++r) sh.G[(f * n + l0) * kM + r] = G2[r];
   }

@@ -142,6 +142,7 @@ struct LimParams {
   int max_iter, fixed_iter;  // Picard of the subcell predictor (as the DG predictor's)
   double tol;
   double gamma, gm1;
+  FxGas gas;
   double delta0, eps;    // NAD tolerances
   StepParams sp;
   OpsD ops;
