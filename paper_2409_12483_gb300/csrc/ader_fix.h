@@ -14,10 +14,13 @@
 // A contraction sum_j c_j x_j keeps two 64-bit sums, hh = sum h h and
 // m = sum (h l + l h); the l l terms (below 2^-2 of the last bit kept, of either
 // sign) are left out.  The value of the sum is hh + m 2^-32 in units of 2^64.
-// All functions also compile for the host (the arithmetic is tested there).
+// All functions also compile for the host (tests/host_src/fixed_check.cpp measures them there).
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
+#include <cstdlib>
 #include <cstring>
 
 #ifdef __CUDACC__
@@ -27,6 +30,12 @@
 #endif
 
 namespace ader {
+
+#ifndef __CUDACC__
+using std::abs;
+using std::max;
+using std::min;
+#endif
 
 typedef long long fxi;
 
@@ -62,6 +71,69 @@ ADER_HD fxi fx_join(unsigned h, unsigned l) {
   return x;
 #else
   return (fxi)(((uint64_t)h << 32) | l);
+#endif
+}
+
+// words of a double, floats and their bits, the float reciprocal within one unit in the
+// last place (any x that is not far from one), leading zeros
+ADER_HD int fx_dhi(double x) {
+#ifdef __CUDA_ARCH__
+  return __double2hiint(x);
+#else
+  uint64_t b;
+  std::memcpy(&b, &x, 8);
+  return (int)(uint32_t)(b >> 32);
+#endif
+}
+ADER_HD int fx_dlo(double x) {
+#ifdef __CUDA_ARCH__
+  return __double2loint(x);
+#else
+  uint64_t b;
+  std::memcpy(&b, &x, 8);
+  return (int)(uint32_t)b;
+#endif
+}
+ADER_HD double fx_double(int hi, int lo) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(hi, lo);
+#else
+  const uint64_t b = (uint64_t)(uint32_t)hi << 32 | (uint32_t)lo;
+  double x;
+  std::memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+ADER_HD unsigned fx_fbits(float x) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(x);
+#else
+  uint32_t b;
+  std::memcpy(&b, &x, 4);
+  return b;
+#endif
+}
+ADER_HD int fx_rint(float x) {
+#ifdef __CUDA_ARCH__
+  return __float2int_rn(x);
+#else
+  return x >= 0x1p31f ? 0x7fffffff : x > -0x1p31f ? (int)lrintf(x) : (int)0x80000000u;
+#endif
+}
+ADER_HD float fx_rcpf(float x) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return 1.0f / x;
+#endif
+}
+ADER_HD int fx_clz(unsigned long long x) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)x);
+#else
+  return x ? __builtin_clzll(x) : 64;
 #endif
 }
 
@@ -140,13 +212,7 @@ ADER_HD void fx_fluxes(const fxi (&q)[D + 2], int g2h, int g2l, fxi (&F)[D][D + 
                        unsigned& bad, Fx2* velocity = nullptr) {
   const Fx2 R = fx_split(q[0]);
   bad |= (unsigned)(R.h - 0x4100000) & 0x80000000u;
-#ifdef __CUDA_ARCH__
-  float rf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"((float)R.h));
-  const int r0 = __float2int_rn(rf * 0x1p57f);  // frac 28
-#else
-  const int r0 = R.h < 0x4100000 ? 0 : (int)(0x1p57f * (1.0f / (float)R.h));
-#endif
+  const int r0 = fx_rint(fx_rcpf((float)R.h) * 0x1p57f);  // frac 28
   const int nh = (int)(0u - (unsigned)R.h);
   const fxi e = fx_madw(nh, r0, (fxi)1 << 57);
   const int es = (int)fx_funnel_l((unsigned)fx_lo(e), (unsigned)fx_hi(e), 24);  // e >> 8

@@ -106,6 +106,7 @@ void split_fx(long double x, int frac, int out[2]);
 bool set_fx_gamma(double gamma, OpsI* o);
 
 // gamma and (gamma - 1) / 2 of an interface kernel; ok: the fixed-point form may run
+// (9/8 <= gamma <= 2)
 struct FxGas {
   int g2h, g2l;  // (gamma - 1) / 2 at frac 62
   int gh, gl;    // gamma at frac 60
