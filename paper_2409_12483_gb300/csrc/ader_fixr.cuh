@@ -155,7 +155,8 @@ ADER_HD fxi fx_sound_speed(fxi rho, fxi p57, int r1, float c0, const FxGas& g, u
 }
 
 // Twice the Rusanov flux between a (low side) and b in direction DIR.  False: not taken
-// (G2 unset).  speed, where asked for: s, the two normal velocities and the bound on the
+// (G2 unset).  speed, where asked for: s (always the refined one: a further variable's jump
+// has nothing to do with the Euler ones), the two normal velocities and the bound on the
 // relative error of s, for further variables' fluxes.
 template <int D, int DIR>
 ADER_HD bool fx_rusanov2(const double* a, const double* b, double* G2, const FxGas& g,
@@ -211,7 +212,7 @@ ADER_HD bool fx_rusanov2(const double* a, const double* b, double* G2, const FxG
   double s_out = 0.0;
   // the FP32 speed: c and the sum are within 2^-21 relative, u and si at their last bits
   float s_err = fmaf(0x1p-21f, sf, 0x1p-27f);
-  if (s_err * jf <= 0x1p-54f * ff) {
+  if (!speed && s_err * jf <= 0x1p-54f * ff) {
     if (!(sf < 15.0f)) return false;
     const int si = fx_rint(sf * 0x1p27f);
 #pragma unroll
@@ -220,7 +221,6 @@ ADER_HD bool fx_rusanov2(const double* a, const double* b, double* G2, const FxG
       const FxAcc t{fx_madw(si, x.h, 0), fx_madw(si, x.l, (fxi)1 << (r < M - 1 ? 30 : 26)), 0};
       sd[r] = r < M - 1 ? fx_fold<1>(t) : fx_fold<5>(t);
     }
-    if (speed) s_out = fx_to_double_int((fxi)si, ec - 27);
   } else {
     // the refined one (fx_sound_speed): its error times the jump below FP64's rounding of the
     // flux, and the jump below 2^-8 of it

@@ -61,10 +61,10 @@ __device__ __forceinline__ void rusanov2_src(const double* a, const double* b, d
   G2[4] = fma(-s, b[4] - a[4], fma(a[4], ua, b[4] * ub));
 }
 
-// The same with the Euler part in fixed point (ader_fixr.cuh) and what it found, the wave
-// speed s and the two velocities, for the other variables: FP64 fluxes q u and s (b - a).
-// False (not taken): the error of s would show beside what the rounding of a and b
-// themselves, 2^-53 each, puts into s (b - a).  Interface kernel of the reacting system,
+// The same with the Euler part in fixed point (ader_fixr.cuh) and what it found, the refined
+// wave speed s (2^-46 or better below Mach 3) and the two velocities, for the other variables:
+// FP64 fluxes q u and s (b - a).  False (not taken): the error of s would show beside what
+// the rounding of a and b themselves, 2^-53 each, puts into s (b - a).  Interface kernel of the reacting system,
 // N = 5, 2e4 cells 34 -> 24 us, of the tracer system (below), N = 3, 2e4 cells 37 -> 19 us;
 // 64 registers instead of 80 measured the same (22.8 and 19.5 us).
 __device__ __forceinline__ bool fx_speed_holds(double a, double b, double d, double err) {

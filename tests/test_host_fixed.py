@@ -42,6 +42,15 @@ def test_rusanov_flux(check, D, slant, gamma, jump):
         assert slant or mach > 300 or jump > 1e-3 or r["taken"] > 4000, (mach, r)
 
 
+@pytest.mark.parametrize("jump", [0.0, 1e-14, 1e-9])
+def test_speed_for_further_variables(check, jump):
+    """refined whatever the Euler jumps are: within 2^-49 + 2^-53 / (c s) of the units (c above
+    2^-12.5, s above 3/16), which is 2^-38 at the most and 2^-46 below Mach 3 (c above 2^-5)"""
+    for mach in MACHS:
+        r = check("flux", 1, 1.4, mach, jump, 0)
+        assert r["rel"] <= (2.0 ** -46 if mach <= 3 else 2.0 ** -38), (mach, r)
+
+
 def test_small_gamma_is_left_to_fp64(check):
     assert check("flux", 1, 1.05, 1.0, 1e-6, 0)["taken"] == 0
 
