@@ -21,8 +21,9 @@
 //
 // Cells whose data do not fit (rho below 1/8 of the cell's power-of-two maximum
 // or not positive, |u| or the iterate beyond twice the cell's units, scales outside
-// 2^+-30, units 2^6 above the slowest cell of the warp, non-finite values) are
-// redone by the FP64 tile code; a cell's result does not depend on the others.
+// 2^+-30, a time step of 2^15 times the CFL limit, non-finite values) are redone by the
+// FP64 tile code.  A cell's result does not depend on the others of its warp or block: the
+// split of a mesh over several contexts (halo cells recomputed) relies on that.
 //
 // Mapping.  A warp holds 32 / n cells, n lanes each; lane p owns the xi node p of
 // every tau row for the point-wise work (flux, time average) and the kappa~
@@ -128,6 +129,20 @@ __device__ __forceinline__ void fx_even_odd(const fxi (&f)[n], Fx2 (&e)[(n + 1) 
     o[k] = fx_split(f[k] - f[n - 1 - k]);
   }
   if (n & 1) e[n / 2] = fx_split(f[n / 2]);
+}
+
+// the limb pairs of a row of nv variables, planes PL apart, by 2^-s (out of line: for the slow
+// cells only)
+template <int n>
+static __device__ __noinline__ void fx_shift_rows(int2* row, int nv, int PL, int s) {
+#pragma unroll 1
+  for (int r = 0; r < nv; ++r)
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+      const int2 v = row[r * PL + k];
+      const Fx2 x = fx_split(fx_shr(((fxi)v.x << 32) + v.y, s));
+      row[r * PL + k] = make_int2(x.h, x.l);
+    }
 }
 
 // A cell the fixed-point form cannot take carries this (not a number the form can
@@ -247,13 +262,14 @@ __device__ __forceinline__ void predict_fix_warp(const PredictParams& P, const T
     }
     __syncwarp();
   } else {
-  // -(dt/dx) kappa~ at frac 62 - ke, so that kappa~ g (g at frac 56 - SK) folds to
-  // frac 57 with a left shift ksh = SK + 3 + ke + ec >= 0 in every cell: ke is the
-  // exponent of dt/dx, raised where the warp's slowest cell needs it
+  // -(dt/dx) kappa~ at frac 62 - ke (ke: the exponent of dt/dx), so that kappa~ g (g at
+  // frac 56 - SK) folds to frac 57 with a left shift ksh = SK + 3 + ke + ec.  A slow cell
+  // (ksh < 0: 4 to 64 times below the fastest by degree, or a small time step) has its g
+  // shifted right by dsh instead: dt/dx is that much smaller against its units, so g's last bit
+  // stays 2^-60 of the result.  Neither depends on the other cells of the warp.
   const int lex = (__double2hiint(lam) >> 20) & 0xfff;  // sign and exponent
-  const int ecmin = __reduce_min_sync(0xffffffffu, valid && !bad ? ec : 1000);
-  const bool lam_ok = lex > 600 && lex < 1400 && ecmin <= 30;
-  const int ke_new = lam_ok ? max(lex - 1022, -(SK + 3) - ecmin) : 0;
+  const bool lam_ok = lex > 600 && lex < 1400;
+  const int ke_new = lam_ok ? lex - 1022 : 0;
   if (ke_new != ke) {  // uniform over the warp
     ke = ke_new;
     const double kscale = lam_ok ? -lam * fx_pow2(62 - ke) : 0.0;
@@ -265,10 +281,13 @@ __device__ __forceinline__ void predict_fix_warp(const PredictParams& P, const T
     }
   }
   int ksh = SK + 3 + ke + ec;
-  if (!lam_ok || ec - ecmin > 6 || (unsigned)ksh > 26u) {
+  if (!lam_ok || ksh > 26) {
     bad = 1u;
     ksh = 0;
   }
+  const int dsh = min(max(-ksh, 0), 62);
+  const bool slow = __any_sync(0xffffffffu, valid && dsh > 0);
+  ksh = max(ksh, 0);
   // rho and m fold 4 bits further, to frac 61; |g| < 2^(59 - ksh) keeps every folded
   // sum below 2^62
   const int gadd = 1 << (27 - ksh);
@@ -320,7 +339,9 @@ __device__ __forceinline__ void predict_fix_warp(const PredictParams& P, const T
         const int2 c = sh.kt[p][k], f = ex[r * PL + k];
         fx_mac(g, c.x, c.y, Fx2{f.x, f.y});
       }
-      const Fx2 gs = fx_split(fx_fold<1>(g));
+      fxi gv = fx_fold<1>(g);
+      if (slow) gv = fx_shr(gv, dsh);
+      const Fx2 gs = fx_split(gv);
       bad |= (unsigned)(gs.h + gadd) & gmask;
       const fxi u = r == 0 ? u0 : r == 1 ? u1 : u2;
       const int sh_r = r < 2 ? ksh + 4 : ksh;
@@ -390,6 +411,7 @@ __device__ __forceinline__ void predict_fix_warp(const PredictParams& P, const T
           }
         }
       }
+      if (slow) fx_shift_rows<n>(row, kM, PL, dsh);
     }
     __syncwarp();
     float dl = 0.0f, qs = 0.0f, sf = sfl;

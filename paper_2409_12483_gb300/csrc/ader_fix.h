@@ -187,6 +187,9 @@ ADER_HD fxi fx_fold_var(const FxAcc& s, int sh, int* top = nullptr) {
                  fx_funnel_l((unsigned)fx_lo(m), w, sh));
 }
 
+// x 2^-s rounded, s in [0, 62] (|x| below 2^61)
+ADER_HD fxi fx_shr(fxi x, int s) { return (x + (((fxi)1 << s) >> 1)) >> s; }
+
 // Formats of the predictor, in the cell's units (|q| < 2): rho and m at frac 61, E
 // at frac 57; fluxes and everything that enters a contraction below 2^60 (frac 57).
 constexpr int kFxF = 57;

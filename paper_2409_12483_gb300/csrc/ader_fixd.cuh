@@ -66,7 +66,7 @@ struct FixDShared {
   int2 kd[D][N + 1][N + 1], vd[D][N + 1][N + 1];  // (dt/h_d) k~ and (dt/h_d) D~ / w
   int2 nk[N + 1][N + 1], nkrow[N + 1];            // -kappa~ and its row sums
   double dt;
-  int go, ecmin;
+  int go;
   int ex[CPB][3];             // largest exponents of rho, the momenta and E
   int ea[CPB], ec[CPB];       // the cell's units
   int bad[CPB];               // the cell goes to the FP64 block code
@@ -97,7 +97,6 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
     double d = 0.0;
     sh.go = predictor_step_dt(P.sp, &d, blockIdx.x == 0) ? 1 : 0;
     sh.dt = d;
-    sh.ecmin = 1000;
   }
   if (tid < CPB) {
     sh.ex[tid][0] = sh.ex[tid][1] = sh.ex[tid][2] = 0;
@@ -158,18 +157,16 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
     sh.ea[tid] = bad ? 0 : ea;
     sh.ec[tid] = bad ? 0 : ec;
     sh.bad[tid] = bad;
-    if ((long long)blockIdx.x * CPB + tid < P.ncells && !bad) atomicMin(&sh.ecmin, ec);
   }
   __syncthreads();
-  // tables at frac 62 - SK - LD - ke: ke the exponent of the largest dt/h_d, raised so
-  // that s folds to frac 58 with a left shift in every cell (see ader_fix.cuh)
+  // tables at frac 62 - SK - LD - ke, ke the exponent of the largest dt/h_d; s folds to
+  // frac 58 with a left shift, a right one in slow cells (see ader_fix.cuh)
   double lmax = lam[0];
 #pragma unroll
   for (int d = 1; d < D; ++d) lmax = lam[d] > lmax ? lam[d] : lmax;
   const int lex = (__double2hiint(lmax) >> 20) & 0xfff;
-  const bool lam_ok = lex > 600 && lex < 1400 && sh.ecmin <= 30;
-  const int ecmin = lam_ok ? sh.ecmin : 0;
-  const int ke = lam_ok ? max(lex - 1022, -(3 + SK + LD) - ecmin) : 0;
+  const bool lam_ok = lex > 600 && lex < 1400;
+  const int ke = lam_ok ? lex - 1022 : 0;
   const double kscale = lam_ok ? fx_pow2(62 - SK - LD - ke) : 0.0;
   for (int i = tid; i < (2 * D + 1) * n * n; i += C::THREADS) {
     const int t = i / (n * n), a = (i / n) % n, b = i % n;
@@ -187,7 +184,7 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
   }
   if (tid < CPB) {
     const int ksh = 3 + SK + LD + ke + sh.ec[tid];
-    if (!lam_ok || sh.ec[tid] - ecmin > 6 || (unsigned)ksh > 26u) sh.bad[tid] = 1;
+    if (!lam_ok || ksh > 26) sh.bad[tid] = 1;
   }
   if (sitem) {
     const int ea = sh.ea[sc], ec = sh.ec[sc];
@@ -198,7 +195,7 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
   }
   __syncthreads();
   // fold of s, its rounding and the check |s| < 2 (frac 58, before the shift)
-  auto fold_of = [&](int c) { return sh.bad[c] ? 0 : 3 + SK + LD + ke + sh.ec[c]; };
+  auto fold_of = [&](int c) { return sh.bad[c] ? 0 : max(3 + SK + LD + ke + sh.ec[c], -62); };
   const int ksh = fold_of(lc), ksh_s = sitem ? fold_of(sc) : 0;
   const float sf1 = fx_pow2f(sh.ec[lc]), sfl = fx_pow2f(sh.ea[lc]) * 0x1p-61f;
   const int cap = P.fixed_iter > 0 ? P.fixed_iter : P.max_iter;
@@ -229,9 +226,10 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
     for (int d = 0; d < D; ++d)
 #pragma unroll
       for (int m = 0; m < n; ++m) c[d][m] = sh.kd[d][id[d]][m];
-    const fxi rnd = (fxi)1 << (31 - sh_s);
-    const int add = 1 << (27 - sh_s);
-    const unsigned mask = ~0u << (28 - sh_s);
+    const int up = max(sh_s, 0);
+    const fxi rnd = (fxi)1 << (31 - up);
+    const int add = 1 << (27 - up);
+    const unsigned mask = ~0u << (28 - up);
     unsigned b = 0u;
 #pragma unroll 1
     for (int r = 0; r < M; ++r) {
@@ -246,11 +244,12 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
         }
       }
       int top;
-      const Fx2 s = fx_split(fx_fold_var(a, sh_s, &top));
+      const Fx2 s = fx_split(fx_fold_var(a, up, &top));
       b |= (unsigned)(top + add) & mask;
       Sp[r * PL + cell0 + nd] = make_int2(s.h, s.l);
     }
     if (b) atomicOr(flag, 1);
+    if (sh_s < 0) fx_shift_rows<1>(Sp + cell0 + nd, M, PL, -sh_s);
   };
   // this thread's part of the maxima of an iteration (rule R3)
   auto report = [&](int it, float dl, float qs, unsigned big) {
@@ -401,9 +400,10 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
   }
   __syncthreads();
   if (sitem && !sh.bad[sc]) {
-    const fxi rnd = (fxi)1 << (31 - ksh_s);
-    const int add = 1 << (27 - ksh_s);
-    const unsigned mask = ~0u << (28 - ksh_s);
+    const int up = max(ksh_s, 0);
+    const fxi rnd = (fxi)1 << (31 - up);
+    const int add = 1 << (27 - up);
+    const unsigned mask = ~0u << (28 - up);
     unsigned b = 0u;
 #pragma unroll 1
     for (int r = 0; r < M; ++r) {
@@ -418,7 +418,8 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
         }
       }
       int top;
-      const fxi x = fx_fold_var(a, ksh_s, &top);  // frac 58
+      fxi x = fx_fold_var(a, up, &top);  // frac 58
+      if (ksh_s < 0) x = fx_shr(x, -ksh_s);
       b |= (unsigned)(top + add) & mask;
       const fxi u = Up[r * UL + sc * NS + sk];
       const fxi v = r < M - 1 ? u + x * 8 : u + ((x + 1) >> 1);
