@@ -14,8 +14,11 @@
 //
 // Units.  rho, m, E as in ader_fix.cuh (|u| < 2 velocity units 2^ec); each further
 // variable has a power of two of its own above its largest value in the cell and is
-// kept at frac 61.  The source's coefficients dx and dx omega^2 (the source enters as
-// dx S beside k~ F, under (dt/dx) kappa~) are two-limb mantissas with an exponent.
+// kept at frac 61.  A species that is zero in the whole cell and has a source goes to the
+// FP64 code: any unit chosen before it has a size costs it digits (in units of 1, c1 from
+// zero by dt c2 came out 1e-14 to 2e-12 off, FP64 4e-16).  The source's coefficients dx and
+// dx omega^2 (the source enters as dx S beside k~ F, under (dt/dx) kappa~) are two-limb
+// mantissas with an exponent.
 #pragma once
 
 #include "ader_fix.cuh"
@@ -160,6 +163,7 @@ __device__ __forceinline__ void predict_fixs_warp(const PredictParams& P, const 
       es[r - 3] = mx[r] ? mx[r] - 1022 : 0;  // all zero: any unit
       out |= abs(es[r - 3]) > 40;
     }
+    if constexpr (kReact) out |= mx[3] ? !mx[4] && P.om2 > 0.0 : mx[4] != 0;
     if (out) {
       bad = 1u;
       ea = ec = es[0] = es[1] = 0;
