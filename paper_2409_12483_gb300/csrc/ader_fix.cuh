@@ -296,7 +296,7 @@ __device__ __forceinline__ void predict_fix_warp(const PredictParams& P, const T
   const float sf1 = fx_pow2f(ec), sfl = fx_pow2f(ea) * 0x1p-61f;
   const int cap = P.fixed_iter > 0 ? P.fixed_iter : P.max_iter;
   const bool fixed = P.fixed_iter > 0;
-  const float tol = P.tolf;
+  const float tol = P.tolf * kFxTol;
 
   bool done = !valid;
   conv = fixed;
@@ -359,7 +359,7 @@ __device__ __forceinline__ void predict_fix_warp(const PredictParams& P, const T
         qm = max(qm, abs(fx_hi(v)));
       }
       // the largest change is in the last tau row (tau increases with p0)
-      dl = fmaxf(dl, fabsf(fmaf((float)fx_hi(x), 0x1p32f, (float)(unsigned)fx_lo(x))) * sf);
+      dl = fmaxf(dl, fx_abs_float(x) * sf);
       qs = fmaxf(qs, (float)qm * (sf * 0x1p32f));
       big |= (unsigned)qm >> (r < 2 ? 30 : 26);
       sf *= r == 0 ? sf1 : sf1 * 16.0f;
@@ -442,7 +442,7 @@ __device__ __forceinline__ void predict_fix_warp(const PredictParams& P, const T
           const fxi d = v - qc[r * PL + p0 * RS];
           qc[r * PL + p0 * RS] = v;
           qm = max(qm, abs(fx_hi(v)));
-          dm = fmaxf(dm, fabsf(fmaf((float)fx_hi(d), 0x1p32f, (float)(unsigned)fx_lo(d))));
+          dm = fmaxf(dm, fx_abs_float(d));
         }
         dl = fmaxf(dl, dm * sf);
         qs = fmaxf(qs, (float)qm * (sf * 0x1p32f));

@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
       const float dl = __uint_as_float(sh.dl[it & 1][lc]), qs = __uint_as_float(sh.qs[it & 1][lc]);
       if (sh.bad[lc]) {
         done = true;
-      } else if (!fixed && dl <= P.tolf * fmaxf(qs, 1.0f)) {
+      } else if (!fixed && dl <= P.tolf * kFxTol * fmaxf(qs, 1.0f)) {
         done = true;
         conv = true;
       }
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
       const int qm = abs(fx_hi(v));
       if (last) sf *= 16.0f * sf1;
       if (r == 1) sf *= sf1;
-      dl = fmaxf(dl, fabsf(fmaf((float)fx_hi(x), 0x1p32f, (float)(unsigned)fx_lo(x))) * sf);
+      dl = fmaxf(dl, fx_abs_float(x) * sf);
       qs = fmaxf(qs, (float)qm * (sf * 0x1p32f));
       big |= (unsigned)qm >> (last ? 26 : 30);
     }
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(FixDCfg<D, N, T>::THREADS, FixDCfg<D, N, T>::M
         const int qm = abs(fx_hi(v));
         if (last) sf *= 16.0f * sf1;
         if (r == 1) sf *= sf1;
-        dl = fmaxf(dl, fabsf(fmaf((float)fx_hi(d), 0x1p32f, (float)(unsigned)fx_lo(d))) * sf);
+        dl = fmaxf(dl, fx_abs_float(d) * sf);
         qs = fmaxf(qs, (float)qm * (sf * 0x1p32f));
         big |= (unsigned)qm >> (last ? 26 : 30);
       }

@@ -224,15 +224,12 @@ __device__ __forceinline__ void predict_fixs_warp(const PredictParams& P, const 
   const float sf1 = fx_pow2f(ec), sfl = fx_pow2f(ea) * 0x1p-61f;
   const int cap = P.fixed_iter > 0 ? P.fixed_iter : P.max_iter;
   const bool fixed = P.fixed_iter > 0;
-  const float tol = P.tolf, inf = __int_as_float(0x7f800000);
+  const float tol = P.tolf * kFxTol, inf = __int_as_float(0x7f800000);
   auto scale_of = [&](int r) {
     return r == 0   ? sfl
            : r == 1 ? sfl * sf1
            : r == 2 ? sfl * sf1 * sf1 * 16.0f
                     : fx_pow2f(r == 3 ? es[0] : es[1]) * 0x1p-61f;
-  };
-  auto as_float = [](fxi d) {
-    return fabsf(fmaf((float)fx_hi(d), 0x1p32f, (float)(unsigned)fx_lo(d)));
   };
 
   bool done = !valid, ok = true;
@@ -301,7 +298,7 @@ __device__ __forceinline__ void predict_fixs_warp(const PredictParams& P, const 
       const fxi d = v - *qp;
       *qp = v;
       qm = max(qm, abs(fx_hi(v)));
-      dm = fmaxf(dm, as_float(d));
+      dm = fmaxf(dm, fx_abs_float(d));
     }
     const float sc = scale_of(r);
     dl = fmaxf(dl, dm * sc);
@@ -409,7 +406,7 @@ __device__ __forceinline__ void predict_fixs_warp(const PredictParams& P, const 
             qm = max(qm, abs(fx_hi(v)));
           }
           const float sc = scale_of(r);
-          dlE = fmaxf(dlE, as_float(x) * sc);
+          dlE = fmaxf(dlE, fx_abs_float(x) * sc);
           qsE = fmaxf(qsE, (float)qm * (sc * 0x1p32f));
           if ((unsigned)qm >> (r == 2 ? 26 : 30)) bad = 1u;
         } else {
@@ -496,7 +493,7 @@ __device__ __forceinline__ void predict_fixs_warp(const PredictParams& P, const 
         float dm = 0.0f;
 #pragma unroll
         for (int p0 = 0; p0 < n; ++p0)
-          dm = fmaxf(dm, as_float(qc[r * PL + p0 * RS] -
+          dm = fmaxf(dm, fx_abs_float(qc[r * PL + p0 * RS] -
                                   reinterpret_cast<const fxi*>(col)[(r - 3) * PL + p0 * RS]));
         dl = fmaxf(dl, dm * scale_of(r));
       }

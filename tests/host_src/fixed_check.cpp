@@ -7,6 +7,7 @@
 //                                  error of the wave speed handed out over its stated bound,
 //                                  and over the speed itself; faces taken
 //   predictor_flux gamma mach      fx_flux against quadruple precision and FP64
+//   magnitude                      the largest relative error of fx_abs_float
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -147,6 +148,15 @@ static int predictor_flux(double gamma, double mach, long n) {
 int main(int argc, char** argv) {
   if (argc == 4 && !std::strcmp(argv[1], "predictor_flux"))
     return predictor_flux(std::atof(argv[2]), std::atof(argv[3]), 10000);
+  if (argc == 2 && !std::strcmp(argv[1], "magnitude")) {
+    double worst = 0;
+    for (int k = 0; k < 62; ++k)
+      for (long long m : {1ll << k, (1ll << k) + 1, (1ll << k) / 3 + 1, (1ll << k) / 7 * 5 + 1})
+        for (long long x : {m, -m})
+          worst = std::max(worst, std::fabs((double)ader::fx_abs_float(x) / (double)m - 1.0));
+    std::printf("worst=%.17g\n", worst);
+    return 0;
+  }
   if (argc != 7 || std::strcmp(argv[1], "flux")) return 1;
   const int D = std::atoi(argv[2]);
   const double gamma = std::atof(argv[3]), mach = std::atof(argv[4]), jump = std::atof(argv[5]);

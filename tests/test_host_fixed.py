@@ -60,3 +60,9 @@ def test_predictor_flux(check, gamma):
     for mach in MACHS:
         r = check("predictor_flux", gamma, mach)
         assert r["taken"] > 4000 and r["fixed"] <= 2 * r["fp64"], (mach, r)
+
+
+def test_magnitude_of_a_change(check):
+    """what the convergence tests compare: every size and either sign, within the float roundings
+    of the two words and of their sum"""
+    assert check("magnitude")["worst"] <= 2.0 ** -23
