@@ -405,14 +405,14 @@ __global__ void __launch_bounds__(SrcCfg<N, CPB>::THREADS)
   predict_src_tile<N, CPB>(P, io, blockIdx.x, dt, smem, sh);
 }
 
-// Interface tile for the reacting system: C cells per 256-thread block (32: the
+// Interface tile for the reacting system: the cells between C faces (see FaceCfg; 32: the
 // five-variable flux arrays and the Euler-part copies fit the 48 KB of static
 // shared memory at every degree).
 template <int N, int C>
 struct FaceSrcShared {
   FaceShared<N, C> base;  // tables, Euler copies of the new state, lambda reduction
-  double G[(C + 1) * (N + 1) * kMR];
-  double Gs[(C + 1) * kMR];
+  double G[C * (N + 1) * kMR];
+  double Gs[C * kMR];
 };
 
 template <int N, int C>

@@ -360,10 +360,10 @@ __global__ void __launch_bounds__(NcCfg<N, CPB>::THREADS)
 template <int N, int C>
 struct FaceNcShared {
   FaceShared<N, C> base;  // tables, Euler copies of the new state, lambda reduction
-  double G[(C + 1) * (N + 1) * kMN];
-  double B[(C + 1) * (N + 1)];
-  double Gs[(C + 1) * kMN];
-  double Bs[C + 1];
+  double G[C * (N + 1) * kMN];
+  double B[C * (N + 1)];
+  double Gs[C * kMN];
+  double Bs[C];
 };
 
 template <int N, int C>
