@@ -52,10 +52,15 @@ typedef enum {
 typedef enum { ADER_SCHEME_DG = 0, ADER_SCHEME_WENO_FV = 1 } ader_scheme;
 
 typedef enum {
-  ADER_PREC_FP64 = 0,            /* FP64 accuracy throughout; the Euler predictors of N >= 1 (3D:
-                                    N <= 4) run their sweeps in fixed point with 57 to 61 fraction bits
-                                    below each cell's largest values (cells that do not fit,
-                                    and gamma > 2, in FP64), rounded to FP64 once */
+  ADER_PREC_FP64 = 0,            /* FP64 accuracy throughout.  For gamma <= 2 the predictors of N >= 1
+                                    (3D: N <= 4), Euler and both further systems, run their
+                                    sweeps in fixed point with 57 to 61 fraction bits below each
+                                    cell's largest values, rounded to FP64 once; cells that do not
+                                    fit run in FP64.  So do, in every precision form, the
+                                    corrector's epilogue, the WENO reconstruction (N = 2, 4) and,
+                                    for 9/8 <= gamma <= 2, the interface fluxes, each below the
+                                    largest values of its cell, stencil or face.  The form to take:
+                                    of the others only ADER_PREC_FP32_INCREMENT is faster */
   ADER_PREC_FP32_PREDICTOR = 1,  /* Picard in FP32, then fp64_sweeps FP64 sweeps; rest FP64 */
   ADER_PREC_FF_PREDICTOR = 2,    /* Picard and predictor epilogue in float-float (~48 bits,
                                     FP32 pipes); corrector and CFL in FP64 */

@@ -80,7 +80,7 @@ __device__ __forceinline__ bool predictor_step_dt(const StepParams& sp, double* 
   }
   DevCtl* c = sp.ctl;
   // every field first, so that a block waits for one round trip to L2, not for one per
-  // field (N = 2, 100 cells: step 11.2 -> 10.9 us)
+  // field (N = 2, 100 cells: step 22.5 -> 21.8 us)
   const int done = *(volatile int*)&c->done;
   const double lam = bitsd(*(volatile unsigned long long*)&c->lam[sp.par]);
   const int st = *(volatile int*)&c->status;

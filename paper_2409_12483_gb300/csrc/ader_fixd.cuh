@@ -9,7 +9,7 @@
 // memory: fluxes and the contracted s as limb pairs, one plane per variable, so that
 // a warp's 8-byte reads are contiguous.  Predictor per launch, FP64 kernel -> this one:
 // 2D N = 5, 160 x 157 cells 3.74 -> 1.17 ms; 2D N = 3, 256^2 2.12 -> 0.70 ms; 2D N = 7,
-// 80^2 2.49 -> 0.78 ms; 3D N = 3, 48 x 47 x 45 25.0 -> 7.17 ms; 3D N = 1, 64^3 2.94 ->
+// 80^2 2.49 -> 0.78 ms; 3D N = 3, 48 x 47 x 45 25.0 -> 7.23 ms; 3D N = 1, 64^3 2.94 ->
 // 0.88 ms; 3D N = 4, 16^3 3.21 -> 1.03 ms.  ncu: multiplier pipe 58-64 % busy, the rest
 // block barriers (a sweep's phases over the spatial nodes leave most of a block idle)
 // and fixed-latency waits; 4 resident blocks of <= 256 threads measured 3-9 % faster

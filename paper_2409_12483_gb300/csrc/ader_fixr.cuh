@@ -5,7 +5,8 @@
 // cycles of a scheduler each; the same in fixed point is ~340 integer and float
 // instructions without any FP64 one.  Interface kernels, FP64 flux -> this one: 1D
 // N = 5, 1e5 cells 63 -> 46 us, N = 7, 1e6 cells 577 -> 307, 2D N = 5, 160^2 141 -> 80,
-// 3D N = 3, 48^3 2.5 -> 0.81 ms.
+// 3D N = 3, 48^3 2.5 -> 0.82 ms (1 to 3 % of it the bounds below and what they need: 1D N = 5
+// in the present tiles 40.1 -> 41.4 us, N = 7 267 -> 272).
 //
 // Units: powers of two above the two states' largest rho, E and |m| (see ader_fix.cuh);
 // fluxes at frac 57, off by 2^-56 of the units (FP64: 2^-53 of every operand).  The

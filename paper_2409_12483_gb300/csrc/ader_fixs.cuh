@@ -9,8 +9,8 @@
 // (N = 5, 10^5 cells: reacting 1.84 ms, tracer 1.34 ms).  Here the source is point-wise
 // and kappa~ runs along tau, so the reacting system's inner loop stays in one lane's
 // column; the tracer's needs the row derivative of phi each time.  Step times (predictor,
-// interface, CFL pass): reacting N = 5, 10^5 cells 1.97 -> 0.62 ms; tracer N = 3, 30011
-// cells 363 -> 122 us per step of a solve.
+// interface, CFL pass): reacting N = 5, 10^5 cells 1.97 -> 0.56 ms; tracer N = 3, 30011
+// cells 363 -> 88 us per step of a solve.
 //
 // Units.  rho, m, E as in ader_fix.cuh (|u| < 2 velocity units 2^ec); each further
 // variable has a power of two of its own above its largest value in the cell and is

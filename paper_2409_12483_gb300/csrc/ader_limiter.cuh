@@ -35,7 +35,7 @@
 // left to one lane that several can share: detectors by (neighbour, subcell,
 // variable), predictor by (subcell, space-time node), fluxes by (face, tau node).
 // Sod tube, N = 3, 10007 cells, per step, against one lane per cell in the detectors and
-// per subcell in the recomputation: detectors 40 -> 10 us, recomputation 67 -> 24, finish
+// per subcell in the recomputation: detectors 40 -> 10 us, recomputation 67 -> 25, finish
 // (which formed the DG fluxes) 31 -> 11; every cell recomputed (mode 2), N = 5, 1e5 cells:
 // step 1.82 -> 1.55 ms.
 //
